@@ -97,11 +97,13 @@ LBM_API int lbm_init_tgv(float* f, lbm_shape s, double rho0, double u0, double k
 
 /* nsteps BGK steps (Eq. 1 with the equilibrium of Eq. 2, Fig. 1 loop):
  * pull-stream with periodic wrap, moments, f^eq, relaxation
- * f* = f - (f - f^eq)/tau, store.  One fused kernel per step.
+ * f* = f - (f - f^eq)/tau, store.  One fused kernel per step, or one for
+ * several (the same arithmetic: the results do not depend on it, bit for bit).
  *   f_in   device, read only; the state after n steps.
  *   f_out  device; receives the state after n + nsteps steps.  != f_in.
  *   f_tmp  device ping-pong buffer of the same shape, required when
- *          nsteps > 1 (else may be NULL); distinct from f_in and f_out.
+ *          nsteps > 1 (else may be NULL); distinct from f_in and f_out;
+ *          contents undefined afterwards.
  *   tau    relaxation time (> 1/2) of every lattice, used when `taus` is NULL.
  *   taus   optional device float[nb]: per-lattice relaxation times.
  *   totals optional device double[5]; if given it is OVERWRITTEN with FP64

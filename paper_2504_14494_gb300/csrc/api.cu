@@ -167,17 +167,12 @@ int lbm_step_bgk(const float* f_in, float* f_out, float* f_tmp, lbm_shape shape,
     return totals ? cuda_status(launch_moments(f_out, s, nullptr, nullptr, nullptr, totals, st))
                   : LBM_OK;
   }
-  // Ping-pong so that the last step lands in f_out: f_in -> (out|tmp) -> ...
-  const float* src = f_in;
-  for (int k = 0; k < nsteps; ++k) {
-    const int left = nsteps - k;  // steps still to do, this one included
-    float* dst = (left % 2 == 1) ? f_out : f_tmp;
-    const bool last = (left == 1);
-    cudaError_t e = launch_bgk_step(src, dst, s, tau, taus, last ? totals : nullptr, st);
-    if (e != cudaSuccess) return LBM_ERR_CUDA;
-    src = dst;
-  }
-  return LBM_OK;
+  if (nsteps == 1)
+    return cuda_status(launch_bgk_step(f_in, f_out, s, tau, taus, totals, st));
+  if (launch_bgk_steps(f_in, f_out, f_tmp, s, tau, taus, nsteps, st) != cudaSuccess)
+    return LBM_ERR_CUDA;
+  return totals ? cuda_status(launch_moments(f_out, s, nullptr, nullptr, nullptr, totals, st))
+                : LBM_OK;
 }
 
 int lbm_step_channel(const float* f_in, float* f_out, float* f_tmp, lbm_shape shape, float tau,
@@ -205,7 +200,16 @@ int lbm_step_channel(const float* f_in, float* f_out, float* f_tmp, lbm_shape sh
                   : LBM_OK;
   }
   const float* src = f_in;
-  for (int k = 0; k < nsteps; ++k) {
+  int done = 0;
+  if (nsteps > 1 && channel_steps_fit(s, nsteps)) {
+    // all steps on chip, but for a last one with totals (by the single-step kernel)
+    done = totals ? nsteps - 1 : nsteps;
+    float* dst = totals ? f_tmp : f_out;
+    if (launch_channel_steps(f_in, dst, s, tau, taus, force_x, done, st) != cudaSuccess)
+      return LBM_ERR_CUDA;
+    src = dst;
+  }
+  for (int k = done; k < nsteps; ++k) {
     const int left = nsteps - k;
     float* dst = (left % 2 == 1) ? f_out : f_tmp;
     if (launch_channel_step(src, dst, s, tau, taus, force_x, left == 1 ? totals : nullptr, st) !=

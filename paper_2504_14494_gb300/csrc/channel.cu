@@ -18,7 +18,7 @@
 // restriction of an m-times refined channel (odd m) that separates the
 // force part of the non-equilibrium populations from the gradient part
 // (channel_restrict_kernel).
-#include "common.cuh"
+#include "collide.cuh"
 #include "gnn.cuh"
 #include "gnn_launch.h"
 #include "launch.h"
@@ -85,24 +85,6 @@ __device__ __forceinline__ void channel_totals(const float (&f)[Q], bool on,
     double acc = 0.0;
     for (int i = 0; i < 8; ++i) acc += red[i][threadIdx.x];
     if (acc != 0.0) atomicAdd(totals + threadIdx.x, acc);
-  }
-}
-
-// f_i - (f_i - f_i^eq(rho, u))/t + (1 - 1/(2t)) w_i [3 (e_i - u) + 9 (e_i.u) e_i].(gx, 0)
-// with u the force-corrected velocity; t is tau (BGK) or tau tau_adj (Eq. 3).
-__device__ __forceinline__ void channel_relax(float (&f)[Q], float t, float gx) {
-  const float rho = ((f[0] + (f[1] + f[3])) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]));
-  const float jx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
-  const float jy = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-  const float inv = 1.0f / rho;
-  const Moments m{rho, (jx + 0.5f * gx) * inv, jy * inv};
-  const float usq15 = 1.5f * (m.ux * m.ux + m.uy * m.uy);
-  const float omega = 1.0f / t, pre = 1.0f - 0.5f * omega;
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const float eu = float(ex(q)) * m.ux + float(ey(q)) * m.uy;
-    const float src = pre * wq(q) * (3.0f * (float(ex(q)) - m.ux) + 9.0f * eu * float(ex(q))) * gx;
-    f[q] = f[q] - omega * (f[q] - feq_i(q, m, usq15)) + src;
   }
 }
 

@@ -12,6 +12,14 @@ cudaError_t launch_bgk_step(const float* fin, float* fout, const Shape& s, float
 cudaError_t launch_bgk_step_rows(const float* fin, float* fout, const Shape& s, float tau,
                                  const float* taus, double* totals, int64_t row0, int64_t row1,
                                  cudaStream_t st);
+// nsteps >= 2 BGK steps with the state kept on chip between steps
+// (multi_step.cu); ftmp: ping-pong buffer as in lbm_step_bgk.
+cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const Shape& s, float tau,
+                             const float* taus, int nsteps, cudaStream_t st);
+// The same for the channel step, for calls that channel_steps_fit() accepts.
+bool channel_steps_fit(const Shape& s, int nsteps);
+cudaError_t launch_channel_steps(const float* fin, float* fout, const Shape& s, float tau,
+                                 const float* taus, float gx, int nsteps, cudaStream_t st);
 cudaError_t launch_moments(const float* f, const Shape& s, float* rho, float* ux, float* uy,
                            double* totals, cudaStream_t st);
 cudaError_t launch_tgv_init(float* f, const Shape& s, double rho0, double u0, double kx,

@@ -1,0 +1,582 @@
+// Several plain steps per launch: the multi-step calls of the BGK step (Eq. 1,
+// Eq. 2, Fig. 1 loop) and of the channel step, with the state kept on chip
+// between the steps.  Every node of every step is computed by the same
+// bgk_collide / channel_relax on the same nine pulled values as in the
+// single-step kernels, so the results are the same bit for bit.
+//
+// Two forms, chosen by estimated time (launch_bgk_steps):
+//
+// resident_steps_kernel -- for small lattices and many steps, which are bound
+// by the latency of one step: one thread-block cluster (1..8 CTAs) per lattice
+// holds the whole lattice in shared memory (two buffers) for all steps of the
+// call; per step a pull from shared memory, the collision, a store to the
+// other buffer (edge rows also to the neighbouring CTAs' halo rows through
+// distributed shared memory) and one cluster barrier.  64^2: 0.75 us a step
+// (4.1 with one launch a step); a 4 x 32 channel: 0.33 (4.1).
+//
+// temporal_steps_kernel -- for larger lattices, which are bound by memory
+// traffic (72 bytes per node and step): T = 2..4 steps per pass over memory.
+// A strip of 64 columns marches down a range of rows; the rows in flight
+// between its T stages stay in registers (and, for small lattices, pass from
+// warp to warp through shared memory).  The strip is 4 columns wider on each
+// side and the range T rows longer on each side than what is stored (both
+// wrap periodically); those are computed redundantly by the neighbours.
+// 4096^2: 70 us a step against 175 (72 bytes per node at HBM's rate: 178) --
+// bound by FP32 issue (about 100 instructions per node and step) and the 1.2
+// times recomputed nodes; 1024^2: 8.4 (10.6); 512^2: 4.2 (6.2); 256^2: 2.6
+// (4.2); three odd 1023 x 517: 12.3 (22.8).  Tried on the way: one thread per
+// node with all stages handed over in shared memory, 119 at 4096^2; 4 columns
+// per lane, 79 to 83 (fewer warps, and the barrier or the registers bind).
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <cooperative_groups.h>
+#include <type_traits>
+
+#include "collide.cuh"
+#include "launch.h"
+
+namespace cg = cooperative_groups;
+
+
+namespace lbmgnn {
+
+namespace {
+
+__device__ __forceinline__ void cp8(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Resident form.  CTA r of the cluster holds rows r R .. min(ny, (r + 1) R) - 1
+// of lattice b as local rows 1..; local rows 0 and rows + 1 are the halo.
+struct ResidentArgs {
+  const float* fin;
+  float* fout;
+  Shape s;
+  float tau;
+  const float* taus;
+  float gx;
+  int nsteps;  // >= 1
+  int rows;    // R: rows per CTA
+};
+
+// KN: nodes per thread.  CH: the channel (bounce-back walls, force gx).
+template <bool CH, int KN>
+__global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, unsigned* stw) {
+  extern __shared__ float sm[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
+  const int nx = a.s.nx, ny = a.s.ny;
+  const int64_t b = blockIdx.x / C, lat = b * ny * nx;
+  const int ya = r * a.rows, rows = min(ny - ya, a.rows);
+  const int pitch = (a.rows + 2) * nx;  // one plane
+  float *cur = sm, *nxt = sm + Q * pitch;
+  // the neighbours (periodic): the CTA holding row ya - 1 and the one holding
+  // row ya + rows, and the local index of the halo row this CTA fills there
+  const int up = r == 0 ? C - 1 : r - 1, dn = r == C - 1 ? 0 : r + 1;
+  const int up_rows = min(ny - up * a.rows, a.rows);
+  const float* fin = a.fin + lat;
+  // own rows and both halo rows
+  for (int i = threadIdx.x; i < (rows + 2) * nx; i += blockDim.x) {
+    const int ly = i / nx, x = i - ly * nx;
+    int y = ya + ly - 1;
+    y = y < 0 ? ny - 1 : (y >= ny ? 0 : y);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      cur[q * pitch + i] = __ldg(
+          fin + q * a.s.ps + checked((int64_t)y * nx + x, 0, (int64_t)ny * nx, stw));
+  }
+  // this thread's nodes: offset of (local row, 0), x -+ 1 with wrap
+  int row0[KN], xc[KN], xl[KN], xr[KN], ly[KN];
+#pragma unroll
+  for (int k = 0; k < KN; ++k) {
+    const int i = threadIdx.x + k * blockDim.x;
+    ly[k] = i < rows * nx ? i / nx : -1;
+    xc[k] = ly[k] < 0 ? 0 : i - ly[k] * nx;
+    row0[k] = (max(ly[k], 0) + 1) * nx;
+    xl[k] = xc[k] == 0 ? nx - 1 : xc[k] - 1;
+    xr[k] = xc[k] == nx - 1 ? 0 : xc[k] + 1;
+  }
+  const float tau = a.taus ? __ldg(a.taus + b) : a.tau;
+  const float omega = 1.0f / tau;
+  float* up_sm = cl.map_shared_rank(sm, up);
+  float* dn_sm = cl.map_shared_rank(sm, dn);
+  if (C == 1) __syncthreads(); else cl.sync();
+
+  for (int step = 0; step < a.nsteps; ++step) {
+    const int nxt_off = (int)(nxt - sm);
+    const bool last = step == a.nsteps - 1;
+#pragma unroll
+    for (int k = 0; k < KN; ++k) {
+      if (ly[k] < 0) continue;
+      float f[Q];
+      const bool lo = CH && ya + ly[k] == 0, hi = CH && ya + ly[k] == ny - 1;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int xs = ex(q) == 0 ? xc[k] : (ex(q) > 0 ? xl[k] : xr[k]);
+        int o = q * pitch + row0[k] - ey(q) * nx + xs;
+        if (ey(q) > 0 && lo) o = opp(q) * pitch + row0[k] + xc[k];  // halfway bounce-back
+        if (ey(q) < 0 && hi) o = opp(q) * pitch + row0[k] + xc[k];
+        f[q] = cur[o];
+      }
+      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide(f, omega);
+      if (last) {
+        float* o = a.fout + lat + (int64_t)(ya + ly[k]) * nx + xc[k];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) o[q * a.s.ps] = f[q];
+      } else {
+        const int o = row0[k] + xc[k];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) nxt[q * pitch + o] = f[q];
+        // the rows the neighbours pull across the cut (the channel's walls
+        // need none, and nothing reads what is stored for them)
+        if (ly[k] == 0) {  // e_y = -1: below the last row of `up`
+          float* h = up_sm + nxt_off + (up_rows + 1) * nx + xc[k];
+          h[4 * pitch] = f[4], h[7 * pitch] = f[7], h[8 * pitch] = f[8];
+        }
+        if (ly[k] == rows - 1) {  // e_y = +1: above the first row of `dn`
+          float* h = dn_sm + nxt_off + xc[k];
+          h[2 * pitch] = f[2], h[5 * pitch] = f[5], h[6 * pitch] = f[6];
+        }
+      }
+    }
+    if (C == 1) __syncthreads(); else cl.sync();
+    float* t = cur;
+    cur = nxt;
+    nxt = t;
+  }
+}
+
+constexpr int SMEM_MAX = 227 * 1024;
+
+uint32_t resident_smem(int rows, int nx) { return 2u * Q * (uint32_t)(rows + 2) * nx * 4u; }
+
+// Cluster size and rows per CTA, or C = 0 when the lattice does not fit.
+struct ResidentPlan {
+  int C, rows, threads, kn;
+};
+ResidentPlan plan_resident(const Shape& s) {
+  ResidentPlan best{0, 0, 0, 0};
+  if ((int64_t)s.nx * s.ny > 8 * 3072) return best;
+  for (int C = 8; C >= 1; C >>= 1) {
+    if (C > s.ny) continue;
+    const int rows = (s.ny + C - 1) / C;
+    if ((int64_t)rows * (C - 1) >= s.ny) continue;  // a CTA without rows
+    if (resident_smem(rows, s.nx) > (uint32_t)SMEM_MAX) break;
+    const int nodes = rows * s.nx;
+    const int kn = (nodes + 1023) / 1024;
+    if (kn > 3) break;
+    const int threads = ((nodes + kn - 1) / kn + 31) / 32 * 32;
+    // keep the largest cluster unless its CTAs would be less than 4 warps
+    if (best.C && best.threads * best.kn >= 128) break;
+    best = {C, rows, threads, kn};
+  }
+  return best;
+}
+
+template <bool CH, int KN>
+cudaError_t resident_t(const ResidentArgs& a, const ResidentPlan& p, cudaStream_t st) {
+  unsigned* stw = status_word();
+  if (!stw) return cudaErrorInvalidDevice;
+  const uint32_t bytes = resident_smem(p.rows, a.s.nx);
+  auto* kern = resident_steps_kernel<CH, KN>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)p.C * (unsigned)a.s.nb);
+  cfg.blockDim = dim3((unsigned)p.threads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)p.C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a, stw);
+}
+
+template <bool CH>
+cudaError_t resident(const ResidentArgs& a, const ResidentPlan& p, cudaStream_t st) {
+  switch (p.kn) {
+    case 1: return resident_t<CH, 1>(a, p, st);
+    case 2: return resident_t<CH, 2>(a, p, st);
+    default: return resident_t<CH, 3>(a, p, st);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Temporal form.  A CTA owns a strip of 64 columns (2 per lane, one packed
+// pair) and a range of rows.  Its T steps are T stages, S of them in each of
+// G = T / S warps: a stage receives the rows of the step before it one after
+// the other, keeps the two rows it still needs in registers, and passes its
+// own row on, in registers to the next stage of its warp or through shared
+// memory to the next warp.
+constexpr int COLS = 64;
+constexpr int HALO = 4;              // columns computed redundantly on each side (>= T)
+constexpr int AHEAD = 2;             // input rows in flight
+constexpr int RING = AHEAD + 1;      // input row ring
+constexpr int ROWF = Q * COLS;       // floats of one row
+
+struct TemporalArgs {
+  const float* fin;
+  float* fout;
+  Shape s;
+  float tau;
+  const float* taus;
+  int strips;                // strips of COLS - 2 HALO columns (the last may be narrower)
+  int segs, height;          // row ranges of `height` rows
+  int64_t units;             // nb * strips * segs
+};
+
+// Strips per CTA (four independent warps when one warp holds all stages) and
+// resident CTAs per SM: 12 warps of 168 registers (all stages in one warp) or
+// 24 warps of 80 (one stage per warp).
+template <int G>
+constexpr int temporal_units() {
+  return G == 1 ? 4 : 1;
+}
+template <int G>
+constexpr int temporal_ctas() {
+  return G == 1 ? 3 : 24 / G;
+}
+
+// Shared memory in rows of ROWF floats: the input ring, then two slots per
+// hand-over between warps, then (!VEC) the row being stored.
+template <int G, bool VEC>
+constexpr int temporal_bytes() {
+  return temporal_units<G>() * (RING + 2 * (G - 1) + (VEC ? 0 : 1)) * ROWF * 4;
+}
+// VEC: nx % 2 == 0 and 8-byte aligned planes (8-byte copies and stores;
+// 16-byte copies, half a warp per plane, took 7 to 45 % longer); otherwise
+// columns move one by one, stores through shared memory.
+template <int T, int S, bool VEC>
+__global__ void __launch_bounds__(32 * (T / S) * temporal_units<T / S>(),
+                                  temporal_ctas<T / S>()) temporal_steps_kernel(
+    TemporalArgs a, unsigned* stw) {
+  constexpr int G = T / S;
+  constexpr int U = temporal_units<G>();
+  extern __shared__ float4 sm4[];
+  const int lane = threadIdx.x & 31, w = G == 1 ? 0 : threadIdx.x >> 5;
+  const int sub = G == 1 ? threadIdx.x >> 5 : 0;
+  float* sm = reinterpret_cast<float*>(sm4) + sub * (temporal_bytes<G, VEC>() / (4 * U));
+  const int64_t unit = (int64_t)blockIdx.x * U + sub;
+  if (unit >= a.units) return;  // (U > 1 only: no block-wide barrier below)
+  const int nx = a.s.nx, ny = a.s.ny;
+  const int seg = (int)(unit % a.segs);
+  const int64_t bs = unit / a.segs;
+  const int strip = (int)(bs % a.strips);
+  const int64_t b = bs / a.strips;
+  const int x0 = strip * (COLS - 2 * HALO), y0 = seg * a.height;
+  const int height = min(a.height, ny - y0);
+  const int K = height + 2 * T;  // input rows 0..K-1: lattice row y0 - T + k (periodic)
+  auto wrap = [](int v, int n) {
+    v %= n;
+    return v < 0 ? v + n : v;
+  };
+  // source columns: 2 consecutive ones (VEC) or lane + 32 j
+  int xs[VEC ? 1 : 2];
+#pragma unroll
+  for (int j = 0; j < (VEC ? 1 : 2); ++j)
+    xs[j] = wrap(x0 - HALO + (VEC ? 2 * lane : lane + 32 * j), nx);
+  int yin = wrap(y0 - T, ny);
+  const float* fin = a.fin + b * ny * nx;
+  const int64_t lat_nodes = (int64_t)ny * nx, ps = a.s.ps;
+  const float om = -(1.0f / (a.taus ? __ldg(a.taus + b) : a.tau));
+  const float2 nomega = make_float2(om, om);
+
+  auto fetch = [&](int k) {  // warp 0: input row k -> ring
+    if (k < K) {
+      float* d = sm + (k % RING) * ROWF;
+      if constexpr (VEC) {
+        const int64_t o = checked((int64_t)yin * nx + xs[0], 0, lat_nodes - 1, stw);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) cp8(d + q * COLS + 2 * lane, fin + q * ps + o);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int64_t o = checked((int64_t)yin * nx + xs[j], 0, lat_nodes, stw);
+#pragma unroll
+          for (int q = 0; q < Q; ++q) cp4(d + q * COLS + lane + 32 * j, fin + q * ps + o);
+        }
+      }
+      yin = yin + 1 == ny ? 0 : yin + 1;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (w == 0) {
+    for (int k = 0; k < AHEAD; ++k) fetch(k);
+  }
+  // hand-over slots into and out of this warp; the row being stored (!VEC)
+  const float* in_slot = sm + (RING + 2 * (w - 1)) * ROWF + 2 * lane;
+  float* out_slot = sm + (RING + 2 * w) * ROWF + 2 * lane;
+  float* stage_out = sm + (RING + 2 * (G - 1)) * ROWF;
+  // where the last stage stores: 2 consecutive columns, or lane + 32 j
+  float* out = a.fout + b * ny * nx + (int64_t)y0 * nx + x0 - HALO;
+  const bool vstore = 2 * lane >= HALO && 2 * lane < COLS - HALO && x0 - HALO + 2 * lane < nx;
+
+  // Per stage, z: the e_y = 0 populations of the row received last; p: the
+  // e_y = +1 populations of the last two rows (all already shifted by e_x).
+  float2 z[S][3], p[S][2][3];
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) z[s][j] = p[s][0][j] = p[s][1][j] = make_float2(0.1f, 0.1f);
+
+  // Iteration i: warp w receives row i - (S + 1) w of its input (row k of
+  // any step is the input row k's lattice row) and each of its stages
+  // computes the row before the one it receives.  PAR = i & 1 selects the
+  // hand-over slots and the p row to replace.
+  auto iteration = [&](int i, auto par) {
+    constexpr int PAR = decltype(par)::value;
+    float2 f[Q][1];
+    if (w == 0) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+      __syncwarp();  // every lane's copies of row i have landed
+    }
+    {
+      const float* r = w == 0 ? sm + (i % RING) * ROWF + 2 * lane : in_slot + (1 - PAR) * ROWF;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) f[q][0] = *reinterpret_cast<const float2*>(r + q * COLS);
+    }
+    if (w == 0) fetch(i + AHEAD);  // into the slot of row i - 1, which every lane has read
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      // shift by e_x (the strip's outer columns take whatever the edge lanes
+      // hold: they are never stored)
+      float2 g[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        g[q] = f[q][0];
+        if (ex(q) > 0)
+          g[q] = make_float2(__shfl_up_sync(0xffffffffu, g[q].y, 1), g[q].x);
+        else if (ex(q) < 0)
+          g[q] = make_float2(g[q].y, __shfl_down_sync(0xffffffffu, g[q].x, 1));
+      }
+      // e_y = -1 from the row just received, e_y = 0 from the one before it,
+      // e_y = +1 from the one before that
+      f[0][0] = z[s][0], f[1][0] = z[s][1], f[3][0] = z[s][2];
+      f[2][0] = p[s][PAR][0], f[5][0] = p[s][PAR][1], f[6][0] = p[s][PAR][2];
+      f[4][0] = g[4], f[7][0] = g[7], f[8][0] = g[8];
+      z[s][0] = g[0], z[s][1] = g[1], z[s][2] = g[3];
+      p[s][PAR][0] = g[2], p[s][PAR][1] = g[5], p[s][PAR][2] = g[6];
+      bgk_collide_pairs(f, nomega);
+    }
+    if (w < G - 1) {
+      float* o = out_slot + PAR * ROWF;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * COLS) = f[q][0];
+    } else if (i >= 2 * T + G - 1) {  // lattice row y0 + i - (2 T + G - 1)
+      float* o = out + (int64_t)(i - (2 * T + G - 1)) * nx;
+      if constexpr (VEC) {
+        if (vstore) {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * ps + 2 * lane) = f[q][0];
+        }
+      } else {
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+          *reinterpret_cast<float2*>(stage_out + q * COLS + 2 * lane) = f[q][0];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int cc = lane + 32 * j;
+          if (cc >= HALO && cc < COLS - HALO && x0 - HALO + cc < nx) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) o[q * ps + cc] = stage_out[q * COLS + cc];
+          }
+        }
+      }
+    }
+    if constexpr (G > 1) __syncthreads();
+  };
+  const int iters = K + G - 1;
+  for (int i = 0; i < iters; i += 2) {
+    iteration(i, std::integral_constant<int, 0>{});
+    if (i + 1 < iters) iteration(i + 1, std::integral_constant<int, 1>{});
+  }
+}
+
+template <int T, int S, bool VEC>
+cudaError_t temporal_t(TemporalArgs a, cudaStream_t st) {
+  constexpr int G = T / S, U = temporal_units<G>();
+  unsigned* stw = status_word();
+  if (!stw) return cudaErrorInvalidDevice;
+  temporal_steps_kernel<T, S, VEC>
+      <<<(unsigned)((a.units + U - 1) / U), 32 * G * U, temporal_bytes<G, VEC>(), st>>>(a, stw);
+  return cudaGetLastError();
+}
+
+// ---- which form -------------------------------------------------------------
+// Estimated times in microseconds, fitted to sweeps of 64^2 .. 4096^2 lattices
+// and stacks on a GB300 (152 SMs): a step of the single-step kernel (4.1 per
+// launch; 7.3e-6 per node out of L2, 10.45e-6 out of HBM), a step of the
+// resident form, and a pass of the temporal form.  They only rank the forms.
+double single_us(const Shape& s) {
+  const double n = (double)s.nb * s.ny * s.nx;
+  return std::max({4.1, 3.0 + 7.3e-6 * n, 10.45e-6 * n});
+}
+
+// `nsteps` steps of the resident form: 4 for the launch; per wave of clusters
+// (about 16 of 8 CTAs run at once) 4 to load and store; per step 0.45 for the
+// cluster barrier and the chain of one node and 0.75e-3 per node of a CTA.
+double resident_us(const Shape& s, const ResidentPlan& p, int nsteps) {
+  const int at_once = 128 / p.C;
+  const double waves = (double)((s.nb + at_once - 1) / at_once);
+  return 4.0 + waves * (4.0 + nsteps * (0.45 + 0.75e-3 * p.rows * s.nx));
+}
+
+struct TemporalPlan {
+  double us = 1e30;  // per pass
+  bool one = false;  // all stages in one warp
+  int strips = 0, segs = 0, height = 0;
+};
+
+// A pass of T steps: 4.5 for the launch and the first row, and per row an
+// iteration whose time depends on the warps that share the SM (one stage per
+// warp: 0.33 alone, 0.89 at 24 warps; four stages in one warp: 0.65 alone,
+// 1.54 at 12), at least what HBM takes for the state once in and out.  The
+// range heights tried are those that give 1, 2, .. CTAs per SM and whole
+// waves: short ranges fill the SMs, long ones recompute fewer rows.
+TemporalPlan plan_temporal(const Shape& s, int T, int sms) {
+  TemporalPlan best;
+  const int strips = (s.nx + COLS - 2 * HALO - 1) / (COLS - 2 * HALO);
+  const int64_t cols = (int64_t)s.nb * strips;
+  for (int form = 0; form < 2; ++form) {
+    const bool one = form == 0;
+    const int most = one ? 12 : 24 / T;           // strips' CTAs (warps) per SM
+    // warps (one) or CTAs per SM aimed at, then two and three whole waves
+    const int step = one ? 4 : 1, tries = most / step + 2;
+    for (int k = 1; k <= tries; ++k) {
+      const int want = k * step <= most ? k * step : (k - most / step + 1) * most;
+      const int64_t segs_want = std::max<int64_t>(1, (int64_t)sms * want / cols);
+      const int h = (int)((s.ny + std::min<int64_t>(segs_want, s.ny) - 1) /
+                          std::min<int64_t>(segs_want, s.ny));
+      const int segs = (s.ny + h - 1) / h;
+      const int64_t n = cols * segs;
+      const double per_sm = (double)((n + sms - 1) / sms);
+      const double waves = std::max(1.0, std::ceil(per_sm / most));
+      const double warps = std::min(per_sm, (double)most) * (one ? 1 : T);
+      const double it = one ? std::max(0.25 + 0.1 * T, 0.25 * T * (0.25 + 0.108 * warps))
+                            : std::max(0.33, 0.22 + 0.0278 * warps);
+      const double us =
+          std::max(4.5 + waves * it * (h + 2 * T + (one ? 0 : T - 1)),
+                   13.5e-6 * (double)s.nb * s.ny * s.nx);  // (HBM)
+      if (us < best.us) best = {us, one, strips, segs, h};
+    }
+  }
+  return best;
+}
+
+template <int T>
+cudaError_t temporal(const float* src, float* dst, const Shape& s, float tau, const float* taus,
+                     const TemporalPlan& p, cudaStream_t st) {
+  const TemporalArgs a{src, dst, s, tau, taus, p.strips, p.segs, p.height,
+                       (int64_t)s.nb * p.strips * p.segs};
+  const bool vec = s.nx % 2 == 0 && s.ps % 2 == 0 && ((uintptr_t)src | (uintptr_t)dst) % 8 == 0;
+  if (p.one) return vec ? temporal_t<T, T, true>(a, st) : temporal_t<T, T, false>(a, st);
+  return vec ? temporal_t<T, 1, true>(a, st) : temporal_t<T, 1, false>(a, st);
+}
+
+int sm_count() {
+  static std::atomic<int> cached[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+}  // namespace
+
+cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const Shape& s, float tau,
+                             const float* taus, int nsteps, cudaStream_t st) {
+  constexpr int MOST = 4;  // steps per pass
+  const int sms = sm_count();
+  if (sms <= 0) return cudaErrorInvalidDevice;
+  // Steps per pass: the fewest microseconds in all, for the last ones (up to
+  // TAIL) exactly, before them passes of the cheapest kind per step.
+  constexpr int TAIL = 12;
+  TemporalPlan plan[MOST + 1];
+  double us[MOST + 1] = {0.0, single_us(s)};
+  int cheapest = 1;
+  const bool wide = s.nx >= (1 << 30) || s.ny >= (1 << 30);  // 32-bit rows and columns
+  for (int T = 2; T <= MOST && T <= nsteps; ++T) {
+    if (!wide) plan[T] = plan_temporal(s, T, sms);
+    us[T] = plan[T].us;
+    if (us[T] / T < us[cheapest] / cheapest) cheapest = T;
+  }
+  int left = nsteps, passes = 0;
+  double total = 0.0;
+  int head = 0;  // passes of `cheapest` steps before the tail
+  if (left > TAIL) {
+    head = (left - TAIL + cheapest - 1) / cheapest;
+    left -= head * cheapest;
+    total += head * us[cheapest];
+  }
+  double cost[TAIL + 1] = {0.0};
+  int first[TAIL + 1] = {0};
+  for (int n = 1; n <= left; ++n) {
+    cost[n] = 1e30;
+    for (int T = 1; T <= MOST && T <= n; ++T)
+      if (cost[n - T] + us[T] < cost[n]) cost[n] = cost[n - T] + us[T], first[n] = T;
+  }
+  total += cost[left];
+  passes = head;
+  for (int n = left; n > 0; n -= first[n]) ++passes;
+
+  const ResidentPlan rp = plan_resident(s);
+  if (rp.C && resident_us(s, rp, nsteps) < total) {
+    const ResidentArgs a{fin, fout, s, tau, taus, 0.0f, nsteps, rp.rows};
+    return resident<false>(a, rp, st);
+  }
+  // ping-pong so that the last pass lands in fout
+  const float* src = fin;
+  for (int k = 0; k < passes; ++k) {
+    const int T = k < head ? cheapest : first[left];
+    if (k >= head) left -= T;
+    float* dst = (passes - k) % 2 == 1 ? fout : ftmp;
+    cudaError_t e = cudaSuccess;
+    switch (T) {
+      case 1: e = launch_bgk_step(src, dst, s, tau, taus, nullptr, st); break;
+      case 2: e = temporal<2>(src, dst, s, tau, taus, plan[2], st); break;
+      case 3: e = temporal<3>(src, dst, s, tau, taus, plan[3], st); break;
+      default: e = temporal<4>(src, dst, s, tau, taus, plan[4], st); break;
+    }
+    if (e != cudaSuccess) return e;
+    src = dst;
+  }
+  return cudaSuccess;
+}
+
+// The channel has the resident form alone; its single-step kernel takes 4.2 a
+// launch, 16.7e-6 per node.
+bool channel_steps_fit(const Shape& s, int nsteps) {
+  const ResidentPlan rp = plan_resident(s);
+  const double single = std::max(4.2, 16.7e-6 * (double)s.nb * s.ny * s.nx);
+  return rp.C != 0 && 1.1 * resident_us(s, rp, nsteps) < 4.0 + nsteps * single;
+}
+
+cudaError_t launch_channel_steps(const float* fin, float* fout, const Shape& s, float tau,
+                                 const float* taus, float gx, int nsteps, cudaStream_t st) {
+  const ResidentPlan rp = plan_resident(s);
+  if (!rp.C) return cudaErrorInvalidValue;
+  const ResidentArgs a{fin, fout, s, tau, taus, gx, nsteps, rp.rows};
+  return resident<true>(a, rp, st);
+}
+
+}  // namespace lbmgnn
