@@ -16,11 +16,11 @@
 // two kernels per round.
 //
 // Weight gradients are contractions over nodes.  Each CTA accumulates them
-// on the tensor cores over all tiles it owns (operands written transposed,
-// nodes along K, into 128-byte swizzled shared memory; FP32 accumulators in
-// tensor memory) and writes one partial row; a final kernel sums the rows in
-// a fixed order.  Bias gradients (column sums) ride along as an extra MMA
-// column of ones.
+// on the tensor cores over all tiles it owns (FP32 accumulators in tensor
+// memory) and writes one partial row; a final kernel sums the rows in a fixed
+// order.  Their operands are the node-major tiles of the other products, read
+// across their rows (umma.cuh, MN-major): no transposed copies.  Bias gradients
+// (column sums) ride along as an extra MMA column of ones.
 #include "gnn.cuh"
 #include "gnn_launch.h"
 
@@ -36,6 +36,24 @@ __device__ __forceinline__ void st_col(uint8_t* op, int R, int row0, int node, c
 #pragma unroll
   for (int c = 0; c < NV; ++c)
     *reinterpret_cast<__nv_bfloat16*>(blk + sw128_off(row0 + c, k)) = __float2bfloat16_rn(v[c]);
+}
+
+// Features f0..f0+31 of node n, BF16 words as they are, into row `row` of an
+// SW128 block.
+__device__ __forceinline__ void copy_row32(uint8_t* blk, int row, int f0,
+                                           const __nv_bfloat16* base, int64_t N, int64_t n) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int chunk = (f0 >> 3) + c;
+    *reinterpret_cast<uint4*>(blk + row * 128 + ((chunk ^ (row & 7)) << 4)) =
+        __ldg(chunk8(base, N, n, f0 + 8 * c));
+  }
+}
+
+// Part [off, off + n) of a partial gradient row set to 0 (a CTA whose
+// tensor-core wait gave up).
+__device__ __forceinline__ void zero_grad(float* g, int off, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) g[off + i] = 0.0f;
 }
 
 #ifndef LBM_BWD_PF
@@ -150,8 +168,8 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
   const float teff = t * tau_adj_of(yv[0], variant);
   const float inv = 1.0f / teff;
   const float scale = 2.0f * wb / (9.0f * (float)N);
-  double lp = 0.0;
-  float dta = 0.0f, dyv[NOUT], d[Q], g[Q];
+  DF ls{0.0f, 0.0f};
+  float dta = 0.0f, dyv[NOUT], d[Q], g[Q], rr[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) d[q] = sdf * yv[1 + q];
   if (variant & VAR_CONSERVATIVE) conserve9(d);
@@ -167,7 +185,11 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
       dt += 0.5f * src;
     }
     const float r = fp - __ldg(tgt + q * s.ps + nn);
-    lp += (double)wb * (double)r * (double)r;
+    rr[q] = r;
+    // wb r^2 as an FP32 pair: the rounding errors of both products are exact
+    const float r2 = r * r, w2 = wb * r2;
+    df_add(ls, w2);
+    ls.lo += fmaf(wb, r2, -w2) + wb * fmaf(r, r, -r2);
     g[q] = scale * r;  // dL/df*
     dta += g[q] * dt;
     if (on && f_pred) f_pred[q * s.ps + n] = fp;
@@ -181,7 +203,15 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
 #pragma unroll
     for (int o = 0; o < NOUT; ++o) dy[o * N + n] = dyv[o];
   }
-  // block reduction of the squared error
+  // block reduction of the squared error: the node's sum was carried in FP32
+  // pairs (about 2^-46 relative; nine FP64 products per node bound the kernel,
+  // 277 us for 4.2 M nodes), in FP64 where it leaves their range
+  double lp = (double)ls.hi + (double)ls.lo;
+  if (!(ls.hi >= 1e-25f && ls.hi < 1e30f)) {
+    lp = 0.0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) lp += (double)wb * (double)rr[q] * (double)rr[q];
+  }
   if (!on) lp = 0.0;
   __shared__ double red[8];
 #pragma unroll
@@ -289,26 +319,31 @@ __global__ void loss_finish_kernel(const double* __restrict__ lossp, int nblk, d
 // Head backward: dh2 = dy W_h (CUDA cores), dW_h and db_h accumulated on the
 // tensor cores: D[o][i] += sum_n dy[n][o] [h2 | 1][n][i].
 namespace hb {
-constexpr uint32_t XT = 0, YT = 32768, WHF = 53248, DYS = 55808, SH = 60928, BYTES = 61056;
+// XT: dy transposed (128 rows, 10 used), H2: h2 node-major, ONE: 16 rows, row 0 ones
+constexpr uint32_t XT = 0, ONE = 32768, H2 = 36864, WHF = 53248, DYS = 55808, SH = 60928,
+                   BYTES = 61056;
 }
 
-__global__ void __launch_bounds__(256, 2) gnn_head_bwd_kernel(
+#ifndef LBM_HB_CTAS
+#define LBM_HB_CTAS 2  // resident CTAs per SM
+#endif
+__global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
     const float* __restrict__ dy, const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh,
     float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
   if (!blob_ok(packed, stw)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + hb::SH);
-  zero_smem(sm, hb::WHF);
+  zero_smem(sm, hb::H2);
   copy_g2s(sm + hb::WHF, packed + K::WHF, 2560);
   __syncthreads();
-  ones_row(sm + hb::YT, 80, 64);
+  ones_row(sm + hb::ONE, 16, 0);
   TcCtx tc;
   tc_setup(sh, tc);
   const float* whf = reinterpret_cast<const float*>(sm + hb::WHF);
   float* dys = reinterpret_cast<float*>(sm + hb::DYS);
   uint8_t* XT = sm + hb::XT;
-  uint8_t* YT = sm + hb::YT;
+  uint8_t* H2 = sm + hb::H2;
   const int node = threadIdx.x & 127, half = threadIdx.x >> 7, f0 = half * 32;
   const uint32_t lb = lane_base(tc.tmem);
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
@@ -332,9 +367,7 @@ __global__ void __launch_bounds__(256, 2) gnn_head_bwd_kernel(
       }
       st_col<NOUT>(XT, 128, 0, node, d);
     }
-    float hv[32];
-    ld_pb32(h2, N, nn, f0, hv);
-    st_col<32>(YT, 80, f0, node, hv);
+    copy_row32(H2, node, f0, h2, N, nn);
     __syncthreads();
     float dv[32];
 #pragma unroll
@@ -348,7 +381,8 @@ __global__ void __launch_bounds__(256, 2) gnn_head_bwd_kernel(
     if (on) st_pf32(dh, N, n, f0, dv);
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
-          umma_128xN(tc.tmem, smem_u32(XT), 16384, smem_u32(YT), 10240, 2, 80, acc);
+          umma_nt(tc.tmem, smem_u32(XT), 16384, smem_u32(H2), 0, 64, 8, acc);
+          umma_128xN(tc.tmem + 64, smem_u32(XT), 16384, smem_u32(sm + hb::ONE), 2048, 2, 16, acc);
         })) {
       ok = false;
       break;
@@ -370,6 +404,7 @@ __global__ void __launch_bounds__(256, 2) gnn_head_bwd_kernel(
       g[P::HEAD_B + o] = u[0];
     }
   }
+  if (!ok) zero_grad(G + (int64_t)blockIdx.x * P::TRAINABLE, P::HEAD_W, NOUT * HID + NOUT);
   tc_teardown(sh, tc);
 }
 
@@ -380,10 +415,11 @@ __global__ void __launch_bounds__(256, 2) gnn_head_bwd_kernel(
 // reduction over each warp's nodes).  Outputs dh_part = dh_out + d[h; a]_h
 // and da = d[h; a]_a (FP32).
 namespace rb1 {
-// U holds [h; a] node-major (A of the z_n recompute) until that MMA is done,
-// then dz node-major (16 KB) and dz transposed (16 KB, 64 rows per K block).
-constexpr uint32_t U = 0, HAT = 32768, WN = 65536, WNT = 81920, BN = 98304, DBR = 98560,
-                   SH = 99584, BYTES = 99712;
+// HA: [h; a] node-major (two SW128 blocks), A of the z_n recompute and, across
+// its rows, of dW_n; DZ: dz node-major, A of d[h; a] and, across its rows, B of
+// dW_n.  W_n [64 out x 128 in] read across its rows is B of d[h; a].
+constexpr uint32_t HA = 0, DZ = 32768, WN = 49152, BN = 65536, DBR = 65792, SH = 66816,
+                   BYTES = 66944;
 }
 #ifndef LBM_RB1_CTAS
 #define LBM_RB1_CTAS 2  // resident CTAs per SM
@@ -400,16 +436,13 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
   const uint8_t* kr = packed + K::round_base(round);
   const bool mlp_only = variant_of(reinterpret_cast<const float*>(packed + K::NORM)) & VAR_MLP_ONLY;
   copy_g2s(sm + rb1::WN, kr + K::WN, 16384);
-  copy_g2s(sm + rb1::WNT, kr + K::WNT, 16384);
   copy_g2s(sm + rb1::BN, kr + K::BN, 256);
   __syncthreads();
   TcCtx tc;
   tc_setup(sh, tc);
   const float* bn = reinterpret_cast<const float*>(sm + rb1::BN);
-  uint8_t* HA = sm + rb1::U;
-  uint8_t* DZ = sm + rb1::U;            // after the z_n MMA
-  uint8_t* DZT = sm + rb1::U + 16384;   // after the z_n MMA
-  uint8_t* HAT = sm + rb1::HAT;
+  uint8_t* HA = sm + rb1::HA;
+  uint8_t* DZ = sm + rb1::DZ;
   const int node = threadIdx.x & 127, half = threadIdx.x >> 7, f0 = half * 32;
   const uint32_t lb = lane_base(tc.tmem);
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
@@ -427,15 +460,8 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
       else if (t < 16) l2_prefetch_nodes(a_in, t - 8, N, 16, m0, N);
       else l2_prefetch_nodes(dh_out, t - 16, N, 16, m0, N);
     }
-    {
-      float v[32];
-      ld_pb32(h_in, N, nn, f0, v);
-      st_row32(HA, node, f0, v);
-      st_col<32>(HAT, 128, f0, node, v);
-      ld_pb32(a_in, N, nn, f0, v);
-      st_row32(HA + 16384, node, f0, v);
-      st_col<32>(HAT, 128, HID + f0, node, v);
-    }
+    copy_row32(HA, node, f0, h_in, N, nn);
+    copy_row32(HA + 16384, node, f0, a_in, N, nn);
     if (!tc_run(sh, tc, stw, [&] {
           umma_128xN(tc.tmem, smem_u32(HA), 16384, smem_u32(sm + rb1::WN), 8192, 2, 64, false);
         })) {
@@ -449,15 +475,13 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
       act_and_grad(dz, bn + f0, 32, false, nullptr, dz);  // GELU'(z_n), packed pairs
 #pragma unroll
       for (int c = 0; c < 32; ++c) dz[c] = (on && !mlp_only) ? dho[c] * dz[c] : 0.0f;
-      // the z_n MMA has read [h; a]: its space now takes dz
       st_row32(DZ, node, f0, dz);
-      st_col<32>(DZT, 64, f0, node, dz);
       dbacc += warp_transpose_sum(dz);
     }
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
-          umma_128xN(tc.tmem, smem_u32(DZ), 0, smem_u32(sm + rb1::WNT), 0, 1, 128, false);
-          umma_128xN(tc.tmem + 128, smem_u32(HAT), 16384, smem_u32(DZT), 8192, 2, 64, acc);
+          umma_nt(tc.tmem, smem_u32(DZ), 0, smem_u32(sm + rb1::WN), 8192, 128, 4, false);
+          umma_tt(tc.tmem + 128, smem_u32(HA), 16384, smem_u32(DZ), 0, 64, 8, acc);
         })) {
       ok = false;
       break;
@@ -493,6 +517,9 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
       for (int q = 0; q < 4; ++q) t += dbr[(hh * 4 + q) * 32 + l];
       g[P::NODE_B + threadIdx.x] = t;
     }
+  } else {
+    zero_grad(G + (int64_t)blockIdx.x * P::TRAINABLE + P::ROUND0 + round * P::ROUND_SIZE,
+              P::NODE_W, P::ROUND_SIZE - P::NODE_W);
   }
   tc_teardown(sh, tc);
 }
@@ -506,8 +533,11 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
 // (= sum dA) on the tensor cores and the W_c columns (sum dc_x, sum dc_y) in
 // registers (butterfly reduction over the warp's nodes).
 namespace rb2 {
-constexpr uint32_t DAB = 0, DABT = 32768, HT = 65536, WABT = 86016, CK = 102400, CKH = 104448,
-                   DCR = 105472, SH = 107520, BYTES = 107648;
+// DAB: [dA | dB] node-major, A of the dh product and, across its rows, of
+// dW_a | dW_b; H: h node-major, B of the latter across its rows; ONE: 16 rows,
+// row 0 ones
+constexpr uint32_t DAB = 0, H = 32768, ONE = 49152, WABT = 53248, CK = 69632, CKH = 71680,
+                   DCR = 72704, SH = 74752, BYTES = 74880;
 }
 #ifndef LBM_RB2_CTAS
 #define LBM_RB2_CTAS 1  // resident CTAs per SM (2 fit; measured slower)
@@ -531,11 +561,11 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + rb2::SH);
   const uint8_t* kr = packed + K::round_base(round);
-  zero_smem(sm + rb2::HT, rb2::WABT - rb2::HT);
+  zero_smem(sm + rb2::ONE, rb2::WABT - rb2::ONE);
   copy_g2s(sm + rb2::WABT, kr + K::WABT, 16384);
   copy_g2s(sm + rb2::CK, kr + K::CK, 2048);
   __syncthreads();
-  ones_row(sm + rb2::HT, 80, 64);
+  ones_row(sm + rb2::ONE, 16, 0);
   {  // c_k as FP16 pairs
     const float* ckf = reinterpret_cast<const float*>(sm + rb2::CK);
     __half2* ckw = reinterpret_cast<__half2*>(sm + rb2::CKH);
@@ -546,8 +576,7 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
   tc_setup(sh, tc);
   const __half2* ckh = reinterpret_cast<const __half2*>(sm + rb2::CKH);
   uint8_t* DAB = sm + rb2::DAB;
-  uint8_t* DABT = sm + rb2::DABT;
-  uint8_t* HT = sm + rb2::HT;
+  uint8_t* H = sm + rb2::H;
   // per chunk: lane l's running sum of value l of [dc_x | dc_y] over this warp's nodes
   float dcacc0 = 0.0f, dcacc1 = 0.0f;
   const int node = threadIdx.x & 127, half = threadIdx.x >> 7, f0 = half * 32;
@@ -624,11 +653,9 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
             v[16 + c] = d * ((c & 1) ? sy.y : sy.x);
           }
         }
-        // node-major dA (A operand of the dh MMA) and its transpose
         *reinterpret_cast<uint4*>(DAB + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gA);
         *reinterpret_cast<uint4*>(DAB + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
             pack_bf16x8(gA + 8);
-        st_col<16>(DABT, 128, c0, node, gA);
         // dc sums over this warp's 32 nodes: lane l gets value l of [dc_x | dc_y]
         const float t = warp_transpose_sum(v);
         if (sc == 0)
@@ -683,18 +710,14 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
         *reinterpret_cast<uint4*>(b1 + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gB);
         *reinterpret_cast<uint4*>(b1 + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
             pack_bf16x8(gB + 8);
-        st_col<16>(DABT, 128, HID + c0, node, gB);
       }
     }
-    {
-      float h[32];
-      ld_pb32(h_in, N, nn, f0, h);
-      st_col<32>(HT, 80, f0, node, h);
-    }
+    copy_row32(H, node, f0, h_in, N, nn);
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
           umma_128xN(tc.tmem, smem_u32(DAB), 16384, smem_u32(sm + rb2::WABT), 8192, 2, 64, false);
-          umma_128xN(tc.tmem + 64, smem_u32(DABT), 16384, smem_u32(HT), 10240, 2, 80, acc);
+          umma_tt(tc.tmem + 64, smem_u32(DAB), 16384, smem_u32(H), 0, 64, 8, acc);
+          umma_tn(tc.tmem + 128, smem_u32(DAB), 16384, smem_u32(sm + rb2::ONE), 2048, 16, 8, acc);
         })) {
       ok = false;
       break;
@@ -738,6 +761,9 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
       const int of = 32 * hh + 16 * sc + (l & 15);
       g[P::EDGE_W + of * 130 + 128 + (l >> 4)] = t;
     }
+  } else {
+    zero_grad(G + (int64_t)blockIdx.x * P::TRAINABLE + P::ROUND0 + round * P::ROUND_SIZE,
+              P::EDGE_W, P::NODE_W);
   }
   tc_teardown(sh, tc);
 }
@@ -749,10 +775,12 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
 // dW2, db2 (rows 0..63) and dW1, db1 (rows 64..127).  Optionally the input
 // gradient dL/df_pre through x_hat (f_i, rho and u = j / rho).
 namespace eb {
-// U holds, one after the other within a tile, g1 node-major (A of the z2
-// MMA), dz2 node-major (A of the dg1 MMA) and the df partial sums.
-constexpr uint32_t U = 0, XT = 16384, YT = 49152, W2 = 69632, W2T = 77824, W1F = 86016,
-                   B1 = 89088, B2 = 89344, NORM = 89600, SH = 89728, BYTES = 89856;
+// Node-major tiles: G1 (A of the z2 product and, across its rows, B of dW2),
+// DZ = [dz2 | dz1] (dz2: A of dg1; both, across their rows, A of the weight
+// gradients); XH: 16 rows x_hat (12), ones (1), 0; DXH: the df partial sums.
+// W2 read across its rows is B of dg1.
+constexpr uint32_t G1 = 0, DZ = 16384, XH = 49152, W2 = 53248, W1F = 61440, B1 = 64512,
+                   B2 = 64768, NORM = 65024, SH = 65152, DXH = 65280, BYTES = DXH + 12288;
 }
 #ifndef LBM_EB_CTAS
 #define LBM_EB_CTAS 2  // resident CTAs per SM
@@ -769,12 +797,11 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + eb::SH);
-  zero_smem(sm + eb::YT, eb::W2 - eb::YT);
+  zero_smem(sm + eb::XH, eb::W2 - eb::XH);
   copy_g2s(sm + eb::W2, packed + K::W2, 8192);
-  copy_g2s(sm + eb::W2T, packed + K::W2T, 8192);
   copy_g2s(sm + eb::W1F, packed + K::W1F, 3712);
   __syncthreads();
-  ones_row(sm + eb::YT, 80, 76);
+  ones_row(sm + eb::XH, 16, NFEAT);
   // 1 / sigma (the forward encoder normalises by this product too), beside
   // the tensor-core context
   float* isg = reinterpret_cast<float*>(sm + eb::SH + 64);
@@ -786,11 +813,10 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
   const float* b1 = reinterpret_cast<const float*>(sm + eb::B1);
   const float* b2 = reinterpret_cast<const float*>(sm + eb::B2);
   const float* nrm = reinterpret_cast<const float*>(sm + eb::NORM);
-  float* dxh = reinterpret_cast<float*>(sm + eb::U);  // after the dg1 MMA
-  uint8_t* G1 = sm + eb::U;
-  uint8_t* DZ2 = sm + eb::U;                           // after the z2 MMA
-  uint8_t* XT = sm + eb::XT;
-  uint8_t* YT = sm + eb::YT;
+  float* dxh = reinterpret_cast<float*>(sm + eb::DXH);
+  uint8_t* G1 = sm + eb::G1;
+  uint8_t* DZ = sm + eb::DZ;
+  uint8_t* XH = sm + eb::XH;
   const int node = threadIdx.x & 127, half = threadIdx.x >> 7, f0 = half * 32;
   const bool relu = variant_of(nrm) & VAR_MLP_ONLY;
   const uint32_t lb = lane_base(tc.tmem);
@@ -834,9 +860,8 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
 #pragma unroll
       for (int c = 0; c < 16; ++c) gp1[c] = __floats2half2_rn(z1[2 * c], z1[2 * c + 1]);
       st_row32(G1, node, f0, g);
-      st_col<32>(YT, 80, f0, node, g);
     }
-    if (half == 0) st_col<NFEAT>(YT, 80, HID, node, xh);
+    if (half == 0) st_col<NFEAT>(XH, 16, 0, node, xh);
     if (!tc_run(sh, tc, stw, [&] {
           umma_128xN(tc.tmem, smem_u32(G1), 0, smem_u32(sm + eb::W2), 0, 1, 64, false);
         })) {
@@ -852,10 +877,9 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
 #pragma unroll
       for (int c = 0; c < 32; ++c) d[c] = on ? g0[c] * d[c] : 0.0f;
     }
-    st_row32(DZ2, node, f0, d);
-    st_col<32>(XT, 128, f0, node, d);
+    st_row32(DZ, node, f0, d);
     if (!tc_run(sh, tc, stw, [&] {
-          umma_128xN(tc.tmem, smem_u32(DZ2), 0, smem_u32(sm + eb::W2T), 0, 1, 64, false);
+          umma_nt(tc.tmem, smem_u32(DZ), 0, smem_u32(sm + eb::W2), 0, 64, 4, false);
         })) {
       ok = false;
       break;
@@ -867,7 +891,7 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
       d[2 * c] *= gp.x;
       d[2 * c + 1] *= gp.y;
     }
-    st_col<32>(XT, 128, HID + f0, node, d);
+    st_row32(DZ + 16384, node, f0, d);
     if (df) {
       float px[NFEAT];
 #pragma unroll
@@ -882,7 +906,8 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
     }
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
-          umma_128xN(tc.tmem + 64, smem_u32(XT), 16384, smem_u32(YT), 10240, 2, 80, acc);
+          umma_tt(tc.tmem + 64, smem_u32(DZ), 16384, smem_u32(G1), 0, 64, 8, acc);
+          umma_tn(tc.tmem + 128, smem_u32(DZ), 16384, smem_u32(XH), 2048, 16, 8, acc);
         })) {
       ok = false;
       break;
@@ -920,19 +945,44 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
         g[P::ENC1_B + row - HID] = u[12];
       }
     }
+  } else {
+    zero_grad(G + (int64_t)blockIdx.x * P::TRAINABLE, 0, P::ROUND0);
   }
   tc_teardown(sh, tc);
 }
 
 // ---------------------------------------------------------------------------
-// Sum of the per-CTA gradient rows in a fixed order.
+// Sum of the per-CTA gradient rows, from the first to the last; every kernel
+// writes its own parameters' columns in as many rows as it has CTAs.  A thread
+// per parameter; bound by the latency of its loads, of which 32 rows are in
+// flight (26 us for 512 rows before, most of them empty; 6 for 128 rows).
 // accumulate: add to the gradient already in grad (the steps of a rollout).
-__global__ void grad_reduce_kernel(const float* __restrict__ G, int rows,
-                                   float* __restrict__ grad, bool accumulate) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+struct GradRows {
+  int enc, edge, node, head;
+};
+__global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict__ G,
+                                                         GradRows rows, float* __restrict__ grad,
+                                                         bool accumulate,
+                                                         const uint8_t* __restrict__ packed) {
+  const int p = blockIdx.x * 64 + threadIdx.x;
   if (p >= P::TRAINABLE) return;
+  int n = rows.enc;
+  if (p >= P::HEAD_W)
+    n = rows.head;
+  else if (p >= P::ROUND0)
+    n = (p - P::ROUND0) % P::ROUND_SIZE < P::NODE_W ? rows.edge : rows.node;
+  // an invalid image: no kernel wrote its rows, the gradient is 0
+  if (__ldg(reinterpret_cast<const unsigned*>(packed + K::MAGIC_SLOT)) != K::MAGIC) n = 0;
+  constexpr int BATCH = 32;
   float acc = 0.0f;
-  for (int r = 0; r < rows; ++r) acc += G[(int64_t)r * P::TRAINABLE + p];
+  for (int r0 = 0; r0 < n; r0 += BATCH) {
+    float v[BATCH];
+#pragma unroll
+    for (int i = 0; i < BATCH; ++i)
+      v[i] = r0 + i < n ? __ldg(G + (int64_t)(r0 + i) * P::TRAINABLE + p) : 0.0f;
+#pragma unroll
+    for (int i = 0; i < BATCH; ++i) acc += v[i];
+  }
   grad[p] = accumulate ? grad[p] + acc : acc;
 }
 
@@ -1021,14 +1071,13 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
   if (!stw) return cudaErrorInvalidDevice;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(bl.G, 0, (size_t)GRAD_ROWS * P::TRAINABLE * sizeof(float), st)) !=
-      cudaSuccess)
-    return e;
+  const GradRows rows{(int)grad_grid(N, LBM_EB_CTAS), (int)grad_grid(N, LBM_RB2_CTAS),
+                      (int)grad_grid(N, LBM_RB1_CTAS), (int)grad_grid(N, LBM_HB_CTAS)};
   // head: dh2 -> dh[0]
   {
     const uint32_t bytes = hb::BYTES + 1024;
     if ((e = set_smem(gnn_head_bwd_kernel, bytes)) != cudaSuccess) return e;
-    gnn_head_bwd_kernel<<<grad_grid(N, 2), 256, bytes, st>>>(bl.dy, bl.h2, bl.dh[0], bl.G, s,
+    gnn_head_bwd_kernel<<<rows.head, 256, bytes, st>>>(bl.dy, bl.h2, bl.dh[0], bl.G, s,
                                                              packed, stw);
   }
   // rounds 2 and 1 (index 1, 0): dh[0] -> dh[1] (part) -> dh[0] (in)
@@ -1039,25 +1088,25 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
     {
       const uint32_t bytes = rb1::BYTES + 1024;
       if ((e = set_smem(gnn_round_bwd1_kernel, bytes)) != cudaSuccess) return e;
-      gnn_round_bwd1_kernel<<<grad_grid(N, LBM_RB1_CTAS), 256, bytes, st>>>(hs[r], as[r], bl.dh[0], bl.dh[1],
-                                                                 bl.da, r, bl.G, s, packed, stw);
+      gnn_round_bwd1_kernel<<<rows.node, 256, bytes, st>>>(hs[r], as[r], bl.dh[0], bl.dh[1], bl.da,
+                                                           r, bl.G, s, packed, stw);
     }
     {
       const uint32_t bytes = rb2::BYTES + 1024;
       auto* kern = bl.walls ? gnn_round_bwd2_kernel<true> : gnn_round_bwd2_kernel<false>;
       if ((e = set_smem(kern, bytes)) != cudaSuccess) return e;
-      kern<<<grad_grid(N, LBM_RB2_CTAS), 256, bytes, st>>>(abs_[r], bl.da, bl.dh[1], hs[r],
+      kern<<<rows.edge, 256, bytes, st>>>(abs_[r], bl.da, bl.dh[1], hs[r],
                                                            bl.dh[0], r, bl.G, s, packed, stw);
     }
   }
   {
     const uint32_t bytes = eb::BYTES + 1024;
     if ((e = set_smem(gnn_encode_bwd_kernel, bytes)) != cudaSuccess) return e;
-    gnn_encode_bwd_kernel<<<grad_grid(N, LBM_EB_CTAS), 256, bytes, st>>>(
+    gnn_encode_bwd_kernel<<<rows.enc, 256, bytes, st>>>(
         bl.f_pre, bl.dh[0], bl.df, bl.G, s, bl.fx, bl.fxs, packed, stw);
   }
-  grad_reduce_kernel<<<(P::TRAINABLE + 255) / 256, 256, 0, st>>>(bl.G, GRAD_ROWS, bl.grad,
-                                                                   bl.accumulate);
+  grad_reduce_kernel<<<(P::TRAINABLE + 63) / 64, 64, 0, st>>>(bl.G, rows, bl.grad, bl.accumulate,
+                                                                packed);
   return cudaGetLastError();
 }
 

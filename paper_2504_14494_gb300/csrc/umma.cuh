@@ -163,6 +163,47 @@ __device__ __forceinline__ void umma_128xN(uint32_t tmem_d, uint32_t a_addr, uin
   }
 }
 
+// ---- operands read across their rows (MN-major) ------------------------------------
+// The same SW128 blocks serve as an operand whose K runs down the rows: a block
+// of R rows x 64 values is then K = R (rows) by 64 values of M or N, so a tile
+// stored [node][feature] is also the transposed operand of a contraction over
+// nodes, without a transposed copy.  Rows stay 128 bytes apart, 8-row groups
+// 1024; `blk` is the distance of the next block of 64 M (or N) values.  16 K
+// steps are 2048 bytes.
+__device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t addr, uint32_t blk) {
+  return (sw128_desc(addr) & ~((uint64_t)0x3FFF << 16)) | (uint64_t)((blk & 0x3FFFFu) >> 4) << 16;
+}
+constexpr uint32_t A_MN = 1u << 15, B_MN = 1u << 16;  // instruction descriptor bits
+
+// D (M x N) (+)= A^T B over `nks` K steps, A and B both MN-major.
+__device__ __forceinline__ void umma_tt(uint32_t tmem_d, uint32_t a_addr, uint32_t a_blk,
+                                        uint32_t b_addr, uint32_t b_blk, int N, int nks,
+                                        bool accumulate) {
+  const uint32_t id = idesc_bf16(128, N) | A_MN | B_MN;
+  for (int ks = 0; ks < nks; ++ks)
+    umma_bf16(tmem_d, sw128_desc_mn(a_addr + ks * 2048, a_blk),
+              sw128_desc_mn(b_addr + ks * 2048, b_blk), id, (accumulate || ks > 0) ? 1u : 0u);
+}
+// The same with B K-major: SW128 blocks of N rows x 64 K at b_addr + kb * b_stride.
+__device__ __forceinline__ void umma_tn(uint32_t tmem_d, uint32_t a_addr, uint32_t a_blk,
+                                        uint32_t b_addr, uint32_t b_stride, int N, int nks,
+                                        bool accumulate) {
+  const uint32_t id = idesc_bf16(128, N) | A_MN;
+  for (int ks = 0; ks < nks; ++ks)
+    umma_bf16(tmem_d, sw128_desc_mn(a_addr + ks * 2048, a_blk),
+              sw128_desc(b_addr + (ks >> 2) * b_stride + (ks & 3) * 32), id,
+              (accumulate || ks > 0) ? 1u : 0u);
+}
+// And with A K-major (blocks of 128 rows x 64 K) and B MN-major.
+__device__ __forceinline__ void umma_nt(uint32_t tmem_d, uint32_t a_addr, uint32_t a_stride,
+                                        uint32_t b_addr, uint32_t b_blk, int N, int nks,
+                                        bool accumulate) {
+  const uint32_t id = idesc_bf16(128, N) | B_MN;
+  for (int ks = 0; ks < nks; ++ks)
+    umma_bf16(tmem_d, sw128_desc(a_addr + (ks >> 2) * a_stride + (ks & 3) * 32),
+              sw128_desc_mn(b_addr + ks * 2048, b_blk), id, (accumulate || ks > 0) ? 1u : 0u);
+}
+
 // D (M = 128) = A * B^T over `nks` K steps of 16, A from tensor memory at
 // tmem_a (8 columns per step), B from one SW128 block of N rows at b_addr.
 __device__ __forceinline__ void umma_128xN_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_addr,
