@@ -261,7 +261,7 @@ LBM_API int lbm_step_gnn(const float* f_in, float* f_out, lbm_shape s, float tau
  * kernel: pull-stream, moments, features, Linear + ReLU twice and the heads
  * on the tensor cores, Eq. 3, store; 72 bytes of memory traffic per node and
  * no workspace.  lbm_step_gnn takes the same kernel for such an image (after
- * reading the variant on the device), at the cost of three more launches
+ * reading the variant on the device), at the cost of two more launches
  * that return at once.  Arguments and results as lbm_step_gnn.  An image of
  * a message-passing network is refused on the device: nothing is written
  * and LBM_ERR_BLOB is raised in the status word. */

@@ -99,8 +99,6 @@ int gnn_pack(const float* params, void* packed, void* stream) {
   LBM_TRACE("gnn_pack");
   if (!params || !packed) return LBM_ERR_ARG;
   if (!aligned(packed, 16)) return LBM_ERR_ARG;
-  if (cudaMemsetAsync(packed, 0, K::TOTAL, static_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return LBM_ERR_CUDA;
   return launch_gnn_pack(params, static_cast<uint8_t*>(packed),
                          static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? LBM_OK
@@ -138,12 +136,11 @@ int lbm_step_gnn(const float* f_in, float* f_out, lbm_shape shape, float tau, co
   __half* b0 = reinterpret_cast<__half*>(h0 + N * 64);
   __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(b0 + N * 64);
   __half* b1 = reinterpret_cast<__half*>(h1 + N * 64);
-  // The paper's Fig. 2 network (MLP-only variant, read from the image on the
-  // device) is stepped by one fused kernel; for it the three kernels below
-  // return at once, for every other network the fused kernel does.
-  if (launch_gnn_mlp_step(f_in, f_out, s, tau, taus, pk, false, st) != cudaSuccess)
+  // The first kernel reads the variant from the image: it makes the whole step
+  // of the paper's Fig. 2 network (MLP-only; the rounds below then return at
+  // once) or the encoder of any other.
+  if (launch_gnn_encode_fused(f_in, f_out, s, tau, taus, pk, h0, b0, st) != cudaSuccess)
     return LBM_ERR_CUDA;
-  if (launch_gnn_encode_fused(f_in, s, pk, h0, b0, st) != cudaSuccess) return LBM_ERR_CUDA;
   RoundLaunch r0;
   r0.h_in = h0;
   r0.ab_in = b0;
@@ -182,8 +179,7 @@ int lbm_step_gnn_mlp(const float* f_in, float* f_out, lbm_shape shape, float tau
   if (!aligned(packed, 16)) return LBM_ERR_ARG;
   if (overlap(f_in, f_bytes(s), f_out, f_bytes(s))) return LBM_ERR_ALIAS;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (launch_gnn_mlp_step(f_in, f_out, s, tau, taus, static_cast<const uint8_t*>(packed), true,
-                          st) != cudaSuccess)
+  if (launch_gnn_mlp_step(f_in, f_out, s, tau, taus, static_cast<const uint8_t*>(packed), st) != cudaSuccess)
     return LBM_ERR_CUDA;
   if (totals) {
     if (cudaMemsetAsync(totals, 0, 5 * sizeof(double), st) != cudaSuccess) return LBM_ERR_CUDA;

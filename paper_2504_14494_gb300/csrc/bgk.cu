@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ 
                                                       float* __restrict__ ux,
                                                       float* __restrict__ uy,
                                                       double* __restrict__ totals, unsigned* stw) {
+  dep_sync();
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool on = n < N;
@@ -271,6 +272,7 @@ cudaError_t launch_tgv_init(float* f, const Shape& s, double rho0, double u0, do
 // Streaming only (pull with periodic wrap): f_out_i(x) = f_in_i(x - e_i).
 __global__ void __launch_bounds__(256) stream_kernel(const float* __restrict__ fin,
                                                      float* __restrict__ fout, Shape s) {
+  dep_sync();
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;

@@ -144,6 +144,7 @@ cudaError_t launch_channel_step(const float* fin, float* fout, const Shape& s, f
 __global__ void __launch_bounds__(256) channel_pull_kernel(const float* __restrict__ fin,
                                                            float* __restrict__ fpre, Shape s,
                                                            unsigned* stw) {
+  dep_sync();
   const NodeIdx i = node_idx(s);
   float f[Q];
   channel_pull(fin, s, i.nn, i.x, i.y, i.lat, f, stw);
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(256) channel_gnn_collide_kernel(
     const float* __restrict__ fpre, const float* __restrict__ y, float* __restrict__ fout,
     Shape s, float tau, const float* __restrict__ taus, float gx,
     const uint8_t* __restrict__ packed, double* __restrict__ totals, unsigned* stw) {
+  dep_sync();
   if (!blob_ok(packed, stw)) return;
   const NodeIdx i = node_idx(s);
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;

@@ -193,4 +193,20 @@ struct Shape {
   int64_t ps;  // plane stride in elements
 };
 
+// ---- kernels of one call that overlap at their seams -------------------------
+// The kernels of a multi-kernel call are launched with programmatic stream
+// serialization (launch_after, launch.h): a kernel starts once every CTA of the
+// one before it has passed dep_sync(), reads what no kernel of the call writes
+// but the one before the last or an earlier call (the weights), sets up, and
+// waits in dep_sync() until the one before it has completed and its writes are
+// visible.  Each kernel passes dep_sync() on every path, before it reads or
+// writes anything else, so that "the one before has completed" holds for all
+// before it.  The first kernel of a call is launched normally.
+__device__ __forceinline__ void dep_sync() {
+#if __CUDA_ARCH__ >= 900
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+
 }  // namespace lbmgnn

@@ -391,6 +391,23 @@ __device__ __forceinline__ void st_pf32(float* base, int64_t N, int64_t n, int f
 
 // NF (16 or 32) values versions of the helpers above.
 template <int NF>
+__device__ __forceinline__ void ld_pf(const float* base, int64_t N, int64_t n, int f0, float* v) {
+#pragma unroll
+  for (int c = 0; c < NF / 4; ++c) {
+    const float4 t = __ldg(chunk4(base, N, n, f0 + 4 * c));
+    v[4 * c] = t.x;
+    v[4 * c + 1] = t.y;
+    v[4 * c + 2] = t.z;
+    v[4 * c + 3] = t.w;
+  }
+}
+template <int NF>
+__device__ __forceinline__ void st_pf(float* base, int64_t N, int64_t n, int f0, const float* v) {
+#pragma unroll
+  for (int c = 0; c < NF / 4; ++c)
+    *chunk4w(base, N, n, f0 + 4 * c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+}
+template <int NF>
 __device__ __forceinline__ void ld_pb(const __nv_bfloat16* base, int64_t N, int64_t n, int f0,
                                       float* v) {
 #pragma unroll
@@ -773,6 +790,10 @@ inline unsigned grid_for(int64_t N, int per_sm) {
   const int64_t cap = (int64_t)num_sms() * per_sm;
   return (unsigned)(ntiles < cap ? ntiles : cap);
 }
+
+// One tile per CTA and at most one CTA per SM: the multi-kernel calls then
+// overlap their kernels' seams (launch_after).
+inline bool tiles_alone(int64_t N) { return (N + TILE - 1) / TILE <= num_sms(); }
 
 template <typename KernelT>
 inline cudaError_t set_smem(KernelT k, uint32_t bytes) {

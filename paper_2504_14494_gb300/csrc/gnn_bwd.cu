@@ -23,6 +23,7 @@
 // (column sums) ride along as an extra MMA column of ones.
 #include "gnn.cuh"
 #include "gnn_launch.h"
+#include "launch.h"
 
 namespace lbmgnn {
 
@@ -38,12 +39,13 @@ __device__ __forceinline__ void st_col(uint8_t* op, int R, int row0, int node, c
     *reinterpret_cast<__nv_bfloat16*>(blk + sw128_off(row0 + c, k)) = __float2bfloat16_rn(v[c]);
 }
 
-// Features f0..f0+31 of node n, BF16 words as they are, into row `row` of an
+// Features f0..f0+NF-1 of node n, BF16 words as they are, into row `row` of an
 // SW128 block.
-__device__ __forceinline__ void copy_row32(uint8_t* blk, int row, int f0,
-                                           const __nv_bfloat16* base, int64_t N, int64_t n) {
+template <int NF>
+__device__ __forceinline__ void copy_row(uint8_t* blk, int row, int f0, const __nv_bfloat16* base,
+                                         int64_t N, int64_t n) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < NF / 8; ++c) {
     const int chunk = (f0 >> 3) + c;
     *reinterpret_cast<uint4*>(blk + row * 128 + ((chunk ^ (row & 7)) << 4)) =
         __ldg(chunk8(base, N, n, f0 + 8 * c));
@@ -138,6 +140,7 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
     const float* __restrict__ gxs, const uint8_t* __restrict__ packed,
     double* __restrict__ lossp, float* __restrict__ dy, float* __restrict__ f_pred,
     const float* __restrict__ lw, unsigned* stw) {
+  dep_sync();
   if (!blob_ok(packed, stw)) {  // no loss from an invalid image: NaN
     if (threadIdx.x == 0) lossp[blockIdx.x] = __longlong_as_double(0x7ff8000000000000LL);
     return;
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(256) gnn_collide_adjoint_kernel(
     const float* __restrict__ g_in, Shape s, float tau, const float* __restrict__ taus,
     const uint8_t* __restrict__ packed, float scale, float* __restrict__ dy,
     float* __restrict__ dfd, unsigned* stw) {
+  dep_sync();
   if (!blob_ok(packed, stw)) return;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(256) gnn_collide_adjoint_kernel(
 __global__ void __launch_bounds__(256) stream_adjoint_sum_kernel(
     const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ out, Shape s,
     unsigned* stw) {
+  dep_sync();
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
@@ -301,18 +306,26 @@ __global__ void __launch_bounds__(256) stream_adjoint_sum_kernel(
 }
 
 // Sum of the per-block squared errors, divided by 9 N (deterministic order).
-__global__ void loss_finish_kernel(const double* __restrict__ lossp, int nblk, double count,
-                                   double* __restrict__ loss) {
-  __shared__ double red[256];
+// One block: 1,024 threads with 8 loads in flight each (34 us for 16,384
+// values with 256 threads and one load at a time).
+__global__ void __launch_bounds__(1024) loss_finish_kernel(const double* __restrict__ lossp,
+                                                           int nblk, double count,
+                                                           double* __restrict__ loss) {
+  dep_sync();
+  __shared__ double red[32];
   double acc = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += lossp[i];
-  red[threadIdx.x] = acc;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < nblk; i += 1024) acc += __ldg(lossp + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    acc = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0) *loss = acc / count;
   }
-  if (threadIdx.x == 0) *loss = red[0] / count;
 }
 
 // ---------------------------------------------------------------------------
@@ -330,6 +343,7 @@ constexpr uint32_t XT = 0, ONE = 32768, H2 = 36864, WHF = 53248, DYS = 55808, SH
 __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
     const float* __restrict__ dy, const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh,
     float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
+  dep_sync();  // before the weights: as a call's first kernel it may follow their pack
   if (!blob_ok(packed, stw)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
@@ -367,7 +381,7 @@ __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
       }
       st_col<NOUT>(XT, 128, 0, node, d);
     }
-    copy_row32(H2, node, f0, h2, N, nn);
+    copy_row<32>(H2, node, f0, h2, N, nn);
     __syncthreads();
     float dv[32];
 #pragma unroll
@@ -429,7 +443,7 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
     const __nv_bfloat16* __restrict__ h_in, const __nv_bfloat16* __restrict__ a_in,
     const float* __restrict__ dh_out, float* __restrict__ dh_part, float* __restrict__ da,
     int round, float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
+  if (!blob_ok(packed, stw)) return dep_sync();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + rb1::SH);
@@ -449,6 +463,7 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
   const int64_t ntiles = (N + TILE - 1) / TILE;
   float dbacc = 0.0f;  // lane l: running sum of dz[f0 + l] over this warp's nodes
   bool first = true, ok = true;
+  dep_sync();
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
@@ -460,8 +475,8 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
       else if (t < 16) l2_prefetch_nodes(a_in, t - 8, N, 16, m0, N);
       else l2_prefetch_nodes(dh_out, t - 16, N, 16, m0, N);
     }
-    copy_row32(HA, node, f0, h_in, N, nn);
-    copy_row32(HA + 16384, node, f0, a_in, N, nn);
+    copy_row<32>(HA, node, f0, h_in, N, nn);
+    copy_row<32>(HA + 16384, node, f0, a_in, N, nn);
     if (!tc_run(sh, tc, stw, [&] {
           umma_128xN(tc.tmem, smem_u32(HA), 16384, smem_u32(sm + rb1::WN), 8192, 2, 64, false);
         })) {
@@ -539,24 +554,28 @@ namespace rb2 {
 constexpr uint32_t DAB = 0, H = 32768, ONE = 49152, WABT = 53248, CK = 69632, CKH = 71680,
                    DCR = 72704, SH = 74752, BYTES = 74880;
 }
-#ifndef LBM_RB2_CTAS
-#define LBM_RB2_CTAS 1  // resident CTAs per SM (2 fit; measured slower)
+#ifndef LBM_RB2_GROUP_A
+#define LBM_RB2_GROUP_A 4  // neighbours whose loads are in flight together, dA side
 #endif
-#ifndef LBM_RB2_GROUP
-#define LBM_RB2_GROUP 4  // neighbours whose loads are in flight together
+#ifndef LBM_RB2_GROUP_B
+#define LBM_RB2_GROUP_B 2  // the same, dB side
 #endif
 
 // WALLS (the channel's graph): an edge whose far node lies beyond a wall
 // (row outside [0, ny)) was left out of the forward's sum and passes no
 // gradient; its neighbour address wraps to a row inside, so loads stay in
 // range.
+// Four threads per node, 16 features each: 16 warps of 128 registers per SM.
+// Bound by the latency of the gathers and of the FP16 chains (FP16 pipe 47 %,
+// issue 45 % with two threads per node at 233 registers: 8 warps); 64 x 256^2
+// training step 11.18 -> 10.85 ms, a step of few tiles 37 -> 31 us per launch.
 template <bool WALLS>
-__global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
+__global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
     const __half* __restrict__ ab, const float* __restrict__ da,
     const float* __restrict__ dh_part, const __nv_bfloat16* __restrict__ h_in,
     float* __restrict__ dh_in, int round, float* __restrict__ G, Shape s,
     const uint8_t* __restrict__ packed, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
+  if (!blob_ok(packed, stw)) return dep_sync();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + rb2::SH);
@@ -577,22 +596,21 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
   const __half2* ckh = reinterpret_cast<const __half2*>(sm + rb2::CKH);
   uint8_t* DAB = sm + rb2::DAB;
   uint8_t* H = sm + rb2::H;
-  // per chunk: lane l's running sum of value l of [dc_x | dc_y] over this warp's nodes
-  float dcacc0 = 0.0f, dcacc1 = 0.0f;
-  const int node = threadIdx.x & 127, half = threadIdx.x >> 7, f0 = half * 32;
+  constexpr int NF = 16;  // features of a thread
+  float dcacc = 0.0f;  // lane l: running sum of value l of [dc_x | dc_y] over this warp's nodes
+  const int node = threadIdx.x & 127, part = threadIdx.x >> 7, f0 = part * NF;
   const uint32_t lb = lane_base(tc.tmem);
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t ntiles = (N + TILE - 1) / TILE;
   bool first = true, ok = true;
+  dep_sync();
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
     const NodeXY p = node_xy(nn, s);
-#pragma unroll 1
-    for (int sc = 0; sc < 2; ++sc) {  // two chunks of 16 features
-      const int c0 = f0 + 16 * sc;
-      const int ch = c0 >> 3;
+    {
+      const int c0 = f0, ch = c0 >> 3;
       // 2 GELU'(z) is evaluated in packed FP16 pairs (z = A + B + c_k is O(1)).
       // dA_j = da_j * sum_k GELU'(z_jk) factors: the sums over k (and their
       // e_kx / e_ky weighted forms) are taken in FP16 and multiplied by da_j
@@ -610,17 +628,17 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
 #pragma unroll
         for (int c = 0; c < 8; ++c) S[c] = Sx[c] = Sy[c] = __float2half2_rn(0.0f);
 #pragma unroll
-        for (int g = 0; g < 8; g += LBM_RB2_GROUP) {  // directions k = g+1 .. g+LBM_RB2_GROUP
-          uint4 bn[LBM_RB2_GROUP][2];
+        for (int g = 0; g < 8; g += LBM_RB2_GROUP_A) {  // directions k = g+1 .. g+LBM_RB2_GROUP_A
+          uint4 bn[LBM_RB2_GROUP_A][2];
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP; ++kk) {
+          for (int kk = 0; kk < LBM_RB2_GROUP_A; ++kk) {
             const int k = g + kk + 1;
             const int64_t j = checked(node_at(p, ex(k), ey(k), s), 0, N, stw);
             bn[kk][0] = __ldg(chunk8(ab, N, j, HID + c0));
             bn[kk][1] = __ldg(chunk8(ab, N, j, HID + c0 + 8));
           }
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP; ++kk) {
+          for (int kk = 0; kk < LBM_RB2_GROUP_A; ++kk) {
             const int k = g + kk + 1;
             const __half2* c_k = ckh + (k - 1) * (HID / 2) + c0 / 2;
             const uint32_t* bw = reinterpret_cast<const uint32_t*>(bn[kk]);
@@ -657,11 +675,7 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
         *reinterpret_cast<uint4*>(DAB + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
             pack_bf16x8(gA + 8);
         // dc sums over this warp's 32 nodes: lane l gets value l of [dc_x | dc_y]
-        const float t = warp_transpose_sum(v);
-        if (sc == 0)
-          dcacc0 += t;
-        else
-          dcacc1 += t;
+        dcacc += warp_transpose_sum(v);
       }
       {  // dB_j over the neighbours i = j - e_k
         uint32_t bj[8];
@@ -675,11 +689,11 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
 #pragma unroll
         for (int c = 0; c < 16; ++c) gB[c] = 0.0f;
 #pragma unroll
-        for (int g = 0; g < 8; g += LBM_RB2_GROUP) {
-          uint4 ai[LBM_RB2_GROUP][2];
-          float4 di[LBM_RB2_GROUP][4];
+        for (int g = 0; g < 8; g += LBM_RB2_GROUP_B) {
+          uint4 ai[LBM_RB2_GROUP_B][2];
+          float4 di[LBM_RB2_GROUP_B][4];
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP; ++kk) {
+          for (int kk = 0; kk < LBM_RB2_GROUP_B; ++kk) {
             const int k = g + kk + 1;
             const int64_t i = checked(node_at(p, -ex(k), -ey(k), s), 0, N, stw);
             ai[kk][0] = __ldg(chunk8(ab, N, i, c0));
@@ -688,7 +702,7 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
             for (int t4 = 0; t4 < 4; ++t4) di[kk][t4] = __ldg(chunk4(da, N, i, c0 + 4 * t4));
           }
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP; ++kk) {
+          for (int kk = 0; kk < LBM_RB2_GROUP_B; ++kk) {
             const int k = g + kk + 1;
             const __half2* c_k = ckh + (k - 1) * (HID / 2) + c0 / 2;
             const uint32_t* aw = reinterpret_cast<const uint32_t*>(ai[kk]);
@@ -712,7 +726,7 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
             pack_bf16x8(gB + 8);
       }
     }
-    copy_row32(H, node, f0, h_in, N, nn);
+    copy_row<NF>(H, node, f0, h_in, N, nn);
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
           umma_128xN(tc.tmem, smem_u32(DAB), 16384, smem_u32(sm + rb2::WABT), 8192, 2, 64, false);
@@ -723,13 +737,13 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
       break;
     }
     first = false;
-    float d[32], dp[32];
-    tmem_ld32(lb + f0, d);
+    float d[NF], dp[NF];
+    tmem_ld<NF>(lb + f0, d);
     if (on) {
-      ld_pf32(dh_part, N, n, f0, dp);
+      ld_pf<NF>(dh_part, N, n, f0, dp);
 #pragma unroll
-      for (int c = 0; c < 32; ++c) d[c] += dp[c];
-      st_pf32(dh_in, N, n, f0, d);
+      for (int c = 0; c < NF; ++c) d[c] += dp[c];
+      st_pf<NF>(dh_in, N, n, f0, d);
     }
     tc_fence_before();
     __syncthreads();
@@ -739,27 +753,25 @@ __global__ void __launch_bounds__(256, LBM_RB2_CTAS) gnn_round_bwd2_kernel(
     float* g = G + (int64_t)blockIdx.x * P::TRAINABLE + P::ROUND0 + round * P::ROUND_SIZE;
     const int o = row & 63;
     const int col_off = row < HID ? 0 : HID;
-    float v[32];
-    tmem_ld32(lb + 64 + f0, v);
-    for (int c = 0; c < 32; ++c) g[P::EDGE_W + o * 130 + col_off + f0 + c] = v[c];
-    if (half == 0) {
+    float v[NF];
+    tmem_ld<NF>(lb + 64 + f0, v);
+    for (int c = 0; c < NF; ++c) g[P::EDGE_W + o * 130 + col_off + f0 + c] = v[c];
+    if (part == 0) {
       float u[16];
       tmem_ld16(lb + 128, u);  // column sum of [dA | dB]
       if (row < HID) g[P::EDGE_B + o] = u[0];
     }
-    // W_c columns: the 4 warps of a feature half hold disjoint node sets;
+    // W_c columns: the 4 warps of a feature part hold disjoint node sets;
     // summed in fixed order.
-    float* dcr = reinterpret_cast<float*>(sm + rb2::DCR);  // [8 warps][2 chunks][32]
+    float* dcr = reinterpret_cast<float*>(sm + rb2::DCR);  // [16 warps][32]
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    dcr[(w * 2 + 0) * 32 + lane] = dcacc0;
-    dcr[(w * 2 + 1) * 32 + lane] = dcacc1;
+    dcr[w * 32 + lane] = dcacc;
     __syncthreads();
     if (threadIdx.x < 128) {
-      const int hh = threadIdx.x >> 6, sc = (threadIdx.x >> 5) & 1, l = threadIdx.x & 31;
+      const int pt = threadIdx.x >> 5, l = threadIdx.x & 31;
       float t = 0.0f;
-      for (int q = 0; q < 4; ++q) t += dcr[((hh * 4 + q) * 2 + sc) * 32 + l];
-      const int of = 32 * hh + 16 * sc + (l & 15);
-      g[P::EDGE_W + of * 130 + 128 + (l >> 4)] = t;
+      for (int q = 0; q < 4; ++q) t += dcr[(pt * 4 + q) * 32 + l];
+      g[P::EDGE_W + (16 * pt + (l & 15)) * 130 + 128 + (l >> 4)] = t;
     }
   } else {
     zero_grad(G + (int64_t)blockIdx.x * P::TRAINABLE + P::ROUND0 + round * P::ROUND_SIZE,
@@ -793,7 +805,7 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
     const float* __restrict__ f_pre, const float* __restrict__ dh0, float* __restrict__ df,
     float* __restrict__ G, Shape s, float fx, const float* __restrict__ fxs,
     const uint8_t* __restrict__ packed, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
+  if (!blob_ok(packed, stw)) return dep_sync();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + eb::SH);
@@ -823,6 +835,7 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t ntiles = (N + TILE - 1) / TILE;
   bool first = true, ok = true;
+  dep_sync();
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
@@ -964,6 +977,7 @@ __global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict
                                                          GradRows rows, float* __restrict__ grad,
                                                          bool accumulate,
                                                          const uint8_t* __restrict__ packed) {
+  dep_sync();
   const int p = blockIdx.x * 64 + threadIdx.x;
   if (p >= P::TRAINABLE) return;
   int n = rows.enc;
@@ -990,6 +1004,7 @@ __global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict
 __global__ void adamw_kernel(float* __restrict__ theta, const float* __restrict__ g,
                              float* __restrict__ m, float* __restrict__ v, float lr, float wd,
                              float b1, float b2, float eps, float bc1, float bc2) {
+  dep_sync();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= P::TRAINABLE) return;
   const float gp = g[p];
@@ -1012,10 +1027,9 @@ cudaError_t launch_collide_loss(const float* f_pre, const float* y, const float*
   *nblk = (int)blocks;
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
-  gnn_collide_loss_kernel<false><<<blocks, 256, 0, st>>>(f_pre, y, tgt, s, tau, taus, 0.0f,
-                                                          nullptr, packed, lossp, dy, f_pred, lw,
-                                                          stw);
-  return cudaGetLastError();
+  const bool early = tiles_alone(N);
+  return launch_after(early, gnn_collide_loss_kernel<false>, blocks, 256, 0, st, f_pre, y, tgt, s, tau, taus,
+                      0.0f, nullptr, packed, lossp, dy, f_pred, lw, stw);
 }
 
 cudaError_t launch_collide_loss_channel(const float* f_pre, const float* y, const float* tgt,
@@ -1028,9 +1042,9 @@ cudaError_t launch_collide_loss_channel(const float* f_pre, const float* y, cons
   *nblk = (int)blocks;
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
-  gnn_collide_loss_kernel<true><<<blocks, 256, 0, st>>>(f_pre, y, tgt, s, tau, taus, gx, gxs,
-                                                         packed, lossp, dy, f_pred, lw, stw);
-  return cudaGetLastError();
+  const bool early = tiles_alone(N);
+  return launch_after(early, gnn_collide_loss_kernel<true>, blocks, 256, 0, st, f_pre, y, tgt, s, tau, taus,
+                      gx, gxs, packed, lossp, dy, f_pred, lw, stw);
 }
 
 cudaError_t launch_collide_adjoint(const float* f_pre, const float* y, const float* f_post,
@@ -1040,9 +1054,9 @@ cudaError_t launch_collide_adjoint(const float* f_pre, const float* y, const flo
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
-  gnn_collide_adjoint_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(
-      f_pre, y, f_post, tgt, g_in, s, tau, taus, packed, scale, dy, dfd, stw);
-  return cudaGetLastError();
+  const bool early = tiles_alone(N);
+  return launch_after(early, gnn_collide_adjoint_kernel, (unsigned)((N + 255) / 256), 256, 0, st, f_pre, y,
+                      f_post, tgt, g_in, s, tau, taus, packed, scale, dy, dfd, stw);
 }
 
 cudaError_t launch_stream_adjoint_sum(const float* a, const float* b, float* out, const Shape& s,
@@ -1050,14 +1064,15 @@ cudaError_t launch_stream_adjoint_sum(const float* a, const float* b, float* out
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
-  stream_adjoint_sum_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(a, b, out, s, stw);
-  return cudaGetLastError();
+  const bool early = tiles_alone(N);
+  return launch_after(early, stream_adjoint_sum_kernel, (unsigned)((N + 255) / 256), 256, 0, st, a, b, out,
+                      s, stw);
 }
 
 cudaError_t launch_loss_finish(const double* lossp, int nblk, double count, double* loss,
                                cudaStream_t st) {
-  loss_finish_kernel<<<1, 256, 0, st>>>(lossp, nblk, count, loss);
-  return cudaGetLastError();
+  const bool early = nblk <= 512;
+  return launch_after(early, loss_finish_kernel, 1, 1024, 0, st, lossp, nblk, count, loss);
 }
 
 static unsigned grad_grid(int64_t N, int per_sm) {
@@ -1071,14 +1086,16 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
   if (!stw) return cudaErrorInvalidDevice;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   cudaError_t e;
-  const GradRows rows{(int)grad_grid(N, LBM_EB_CTAS), (int)grad_grid(N, LBM_RB2_CTAS),
+  const bool early = tiles_alone(N);
+  const GradRows rows{(int)grad_grid(N, LBM_EB_CTAS), (int)grad_grid(N, 1),
                       (int)grad_grid(N, LBM_RB1_CTAS), (int)grad_grid(N, LBM_HB_CTAS)};
   // head: dh2 -> dh[0]
   {
     const uint32_t bytes = hb::BYTES + 1024;
     if ((e = set_smem(gnn_head_bwd_kernel, bytes)) != cudaSuccess) return e;
-    gnn_head_bwd_kernel<<<rows.head, 256, bytes, st>>>(bl.dy, bl.h2, bl.dh[0], bl.G, s,
-                                                             packed, stw);
+    if ((e = launch_after(early, gnn_head_bwd_kernel, rows.head, 256, bytes, st, bl.dy, bl.h2, bl.dh[0],
+                          bl.G, s, packed, stw)) != cudaSuccess)
+      return e;
   }
   // rounds 2 and 1 (index 1, 0): dh[0] -> dh[1] (part) -> dh[0] (in)
   const __nv_bfloat16* hs[2] = {bl.h0, bl.h1};
@@ -1088,33 +1105,34 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
     {
       const uint32_t bytes = rb1::BYTES + 1024;
       if ((e = set_smem(gnn_round_bwd1_kernel, bytes)) != cudaSuccess) return e;
-      gnn_round_bwd1_kernel<<<rows.node, 256, bytes, st>>>(hs[r], as[r], bl.dh[0], bl.dh[1], bl.da,
-                                                           r, bl.G, s, packed, stw);
+      if ((e = launch_after(early, gnn_round_bwd1_kernel, rows.node, 256, bytes, st, hs[r], as[r], bl.dh[0],
+                            bl.dh[1], bl.da, r, bl.G, s, packed, stw)) != cudaSuccess)
+        return e;
     }
     {
       const uint32_t bytes = rb2::BYTES + 1024;
       auto* kern = bl.walls ? gnn_round_bwd2_kernel<true> : gnn_round_bwd2_kernel<false>;
       if ((e = set_smem(kern, bytes)) != cudaSuccess) return e;
-      kern<<<rows.edge, 256, bytes, st>>>(abs_[r], bl.da, bl.dh[1], hs[r],
-                                                           bl.dh[0], r, bl.G, s, packed, stw);
+      if ((e = launch_after(early, kern, rows.edge, 512, bytes, st, abs_[r], bl.da, bl.dh[1],
+                            hs[r], bl.dh[0], r, bl.G, s, packed, stw)) != cudaSuccess)
+        return e;
     }
   }
   {
     const uint32_t bytes = eb::BYTES + 1024;
     if ((e = set_smem(gnn_encode_bwd_kernel, bytes)) != cudaSuccess) return e;
-    gnn_encode_bwd_kernel<<<rows.enc, 256, bytes, st>>>(
-        bl.f_pre, bl.dh[0], bl.df, bl.G, s, bl.fx, bl.fxs, packed, stw);
+    if ((e = launch_after(early, gnn_encode_bwd_kernel, rows.enc, 256, bytes, st, bl.f_pre, bl.dh[0], bl.df,
+                          bl.G, s, bl.fx, bl.fxs, packed, stw)) != cudaSuccess)
+      return e;
   }
-  grad_reduce_kernel<<<(P::TRAINABLE + 63) / 64, 64, 0, st>>>(bl.G, rows, bl.grad, bl.accumulate,
-                                                                packed);
-  return cudaGetLastError();
+  return launch_after(early, grad_reduce_kernel, (P::TRAINABLE + 63) / 64, 64, 0, st, bl.G, rows, bl.grad,
+                      bl.accumulate, packed);
 }
 
 cudaError_t launch_adamw(float* theta, const float* g, float* m, float* v, float lr, float wd,
                          float b1, float b2, float eps, float bc1, float bc2, cudaStream_t st) {
-  adamw_kernel<<<(P::TRAINABLE + 255) / 256, 256, 0, st>>>(theta, g, m, v, lr, wd, b1, b2, eps,
-                                                           bc1, bc2);
-  return cudaGetLastError();
+  return launch_after(true, adamw_kernel, (P::TRAINABLE + 255) / 256, 256, 0, st, theta, g, m, v, lr, wd,
+                      b1, b2, eps, bc1, bc2);
 }
 
 }  // namespace lbmgnn

@@ -17,6 +17,7 @@
 // The training forward (gnn_forward) stores A | B ([N][128]) for the backward.
 #include "gnn.cuh"
 #include "gnn_launch.h"
+#include "launch.h"
 
 #ifndef LBM_PREFETCH
 #define LBM_PREFETCH 1  // load the next tile's inputs while computing this one
@@ -32,9 +33,14 @@ __device__ __forceinline__ void put_sw(uint8_t* blk, int row, int k, float v) {
 
 __global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict__ out,
                                 unsigned* stw) {
+  dep_sync();
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
   float* w1f = reinterpret_cast<float*>(out + K::W1F);
+  // the image's unused bytes
+  for (int e = tid; e < 208; e += nth) reinterpret_cast<float*>(out + K::WHF)[NOUT * HID + e] = 0.0f;
+  for (int e = tid; e < 256; e += nth)
+    reinterpret_cast<float*>(out + K::round_base(e >> 7) + K::BN)[HID + (e & 127)] = 0.0f;
   for (int e = tid; e < HID * NFEAT; e += nth) w1f[e] = bf16_round(p[P::ENC1_W + e]);
   for (int e = tid; e < HID; e += nth) {
     reinterpret_cast<float*>(out + K::B1)[e] = p[P::ENC1_B + e];
@@ -65,7 +71,10 @@ __global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict
     reinterpret_cast<float*>(out + K::BH)[e] = e < NOUT ? p[P::HEAD_B + e] : 0.0f;
   for (int e = tid; e < NOUT * HID; e += nth)
     reinterpret_cast<float*>(out + K::WHF)[e] = bf16_round(p[P::HEAD_W + e]);
-  for (int e = tid; e < HID * HID; e += nth) {
+  // the 4,096-element blocks go to threads of their own (64 blocks of 256: a
+  // thread then walks through one of them, not through all)
+  auto at = [&](int section) { return (tid + nth - section * HID * HID % nth) % nth; };
+  for (int e = at(1); e < HID * HID; e += nth) {
     const int o = e / HID, i = e % HID;
     const float w = p[P::ENC2_W + o * HID + i];
     put_sw(out + K::W2, o, i, w);
@@ -75,7 +84,7 @@ __global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict
     const int o = e / HID, i = e % HID;
     put_sw(out + K::WH, o, i, o < NOUT ? p[P::HEAD_W + o * HID + i] : 0.0f);
   }
-  for (int e = tid; e < HID * HID; e += nth) {
+  for (int e = at(2); e < HID * HID; e += nth) {
     const int o = e / HID, k = e % HID;
     const int j = k < 16 ? k : k - 16;
     const float w = (k < 32 && j < NFEAT) ? p[P::ENC1_W + o * NFEAT + j] : 0.0f;
@@ -86,7 +95,7 @@ __global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict
     uint8_t* kr = out + K::round_base(r);
     const float* we = pr + P::EDGE_W;  // [64][130]
     const float* wn = pr + P::NODE_W;  // [64][128]
-    for (int e = tid; e < HID * HID; e += nth) {
+    for (int e = at(3 + r); e < HID * HID; e += nth) {
       const int o = e / HID, i = e % HID;
       const float wa = we[o * 130 + i], wb = we[o * 130 + HID + i];
       put_sw(kr + K::WAB, o, i, wa);
@@ -137,10 +146,7 @@ template <bool PULL, bool BONLY, class Geo>
 __global__ void __launch_bounds__(256, (enc_ctas<PULL, BONLY, Geo>())) gnn_encode_kernel(
     const float* __restrict__ f, Geo geo, const uint8_t* __restrict__ packed,
     __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ ab_out, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
-  if (PULL && BONLY &&
-      (variant_of(reinterpret_cast<const float*>(packed + K::NORM)) & VAR_MLP_ONLY))
-    return;  // inference step of the MLP-only network: the fused kernel (gnn_mlp.cu) did it
+  if (!blob_ok(packed, stw)) return dep_sync();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + enc::SH);
@@ -182,6 +188,7 @@ __global__ void __launch_bounds__(256, (enc_ctas<PULL, BONLY, Geo>())) gnn_encod
     }
   };
   float fnext[Q];
+  dep_sync();
   if (blockIdx.x < ntiles) load_f(blockIdx.x, fnext);
 
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -309,13 +316,17 @@ struct RoundArgs {
 // columns.  In a group, TPN threads per node each own FPT = 64 / TPN
 // features; warp w reads tensor-memory lanes 32 (w % 4)..  AH: the edge
 // terms come as B alone and A = W_a h is computed here from h.
+template <int TPN>
+constexpr int round_ctas() {  // resident CTAs per SM
+  return TPN == 4 ? 1 : LBM_ROUND_CTAS;
+}
 template <int MODE, int TPN, int NG, bool AH, class Geo>
-__global__ void __launch_bounds__(128 * TPN * NG, LBM_ROUND_CTAS) gnn_round_kernel(
+__global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_kernel(
     RoundArgs ra, Geo geo, const uint8_t* __restrict__ packed, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
+  if (!blob_ok(packed, stw)) return dep_sync();
   if ((MODE == 0 || MODE == 1) && ra.h_skip &&
       (variant_of(reinterpret_cast<const float*>(packed + K::NORM)) & VAR_MLP_ONLY))
-    return;  // MLP-only network: no rounds; its inference step is the fused kernel (gnn_mlp.cu)
+    return dep_sync();  // MLP-only network: no rounds; its inference step is the fused kernel (gnn_mlp.cu)
   constexpr int FPT = HID / TPN;
   constexpr int SL = FPT < 32 ? FPT : 32;  // feature slice of the epilogues
   constexpr int GT = 128 * TPN;            // threads per group
@@ -375,6 +386,7 @@ __global__ void __launch_bounds__(128 * TPN * NG, LBM_ROUND_CTAS) gnn_round_kern
 #pragma unroll
     for (int c = 0; c < FPT / 8; ++c) hnext[c] = __ldg(chunk8(h_src, N, mm, f0 + 8 * c));
   };
+  dep_sync();
   if (AH && first < ntiles) load_h(first);
 
   for (int64_t tile = first; tile < ntiles; tile += stride) {
@@ -578,8 +590,7 @@ __global__ void __launch_bounds__(128 * TPN * NG, LBM_ROUND_CTAS) gnn_round_kern
 cudaError_t launch_gnn_pack(const float* params, uint8_t* packed, cudaStream_t st) {
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
-  gnn_pack_kernel<<<64, 256, 0, st>>>(params, packed, stw);
-  return cudaGetLastError();
+  return launch_after(true, gnn_pack_kernel, 64, 256, 0, st, params, packed, stw);
 }
 
 
@@ -609,39 +620,49 @@ static cudaError_t encode_any(const float* f, bool pull, bool b_only, const Geo&
                 : encode_t<false, false>(f, geo, N, per_sm, bytes, packed, h0, ab, stw, st);
 }
 
-template <int MODE, bool AH, class Geo>
-static cudaError_t round_t(const RoundArgs& ra, const Geo& geo, unsigned grid,
-                           const uint8_t* packed, unsigned* stw, cudaStream_t st) {
-  constexpr int T = LBM_ROUND_TPN, G = LBM_ROUND_GROUPS;
+template <int MODE, int T, int G, bool AH, class Geo>
+static cudaError_t round_launch(const RoundArgs& ra, const Geo& geo, unsigned grid,
+                                const uint8_t* packed, unsigned* stw, cudaStream_t st) {
   const uint32_t bytes = RndL<G>::BYTES + 1024;
   cudaError_t e;
   if ((e = set_smem(gnn_round_kernel<MODE, T, G, AH, Geo>, bytes)) != cudaSuccess) return e;
-  gnn_round_kernel<MODE, T, G, AH, Geo><<<grid, 128 * T * G, bytes, st>>>(ra, geo, packed, stw);
-  return cudaGetLastError();
+  return launch_after(T == 4, gnn_round_kernel<MODE, T, G, AH, Geo>, grid, 128 * T * G, bytes, st, ra, geo,
+                      packed, stw);
 }
 
+// Threads per node and tiles per CTA by the number of tiles.  While every tile
+// can have an SM (or half of one) to itself the kernel takes as long as one
+// tile, and four (two) threads per node shorten that; with more tiles than
+// that, one thread per node and four tiles per SM have the higher rate (1024^2
+// step: 0.55 ms, two threads per node 0.58).
+template <int MODE, bool AH, class Geo>
+static cudaError_t round_t(const RoundArgs& ra, const Geo& geo, int64_t N, int per_sm,
+                           const uint8_t* packed, unsigned* stw, cudaStream_t st) {
+  const int64_t ntiles = (N + TILE - 1) / TILE;
+  if (ntiles <= num_sms())
+    return round_launch<MODE, 4, 1, AH>(ra, geo, (unsigned)ntiles, packed, stw, st);
+  if (ntiles <= 2 * num_sms())
+    return round_launch<MODE, 2, 1, AH>(ra, geo, (unsigned)ntiles, packed, stw, st);
+  // persistent grid: at most per_sm CTAs per SM, each running LBM_ROUND_GROUPS tiles at a time
+  const int64_t cta_tiles = (ntiles + LBM_ROUND_GROUPS - 1) / LBM_ROUND_GROUPS;
+  const unsigned grid = grid_for(cta_tiles * TILE, per_sm >= 2 ? LBM_ROUND_CTAS : per_sm);
+  return round_launch<MODE, LBM_ROUND_TPN, LBM_ROUND_GROUPS, AH>(ra, geo, grid, packed, stw, st);
+}
+
+static RoundArgs round_args(const RoundLaunch& rl) {
+  return {rl.h_in, rl.ab_in, rl.h_out, rl.a_out, rl.ab_out, rl.y_out, rl.f_post, rl.f_out,
+          rl.tau, rl.taus, rl.round, rl.h_skip};
+}
+
+// The rounds of an inference step (A recomputed from h): inner round, last
+// round + head + Eq. 3.
 template <class Geo>
-static cudaError_t round_any(int mode, const RoundLaunch& rl, const Geo& geo, int64_t N,
-                             const uint8_t* packed, cudaStream_t st, int per_sm = 2) {
+static cudaError_t round_step(int mode, const RoundLaunch& rl, const Geo& geo, int64_t N,
+                              const uint8_t* packed, cudaStream_t st, int per_sm = 2) {
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
-  // persistent grid: at most per_sm CTAs per SM, each running LBM_ROUND_GROUPS tiles at a time
-  const int64_t cta_tiles = (N + (int64_t)TILE * LBM_ROUND_GROUPS - 1) / ((int64_t)TILE * LBM_ROUND_GROUPS);
-  const unsigned grid = grid_for(cta_tiles * TILE, per_sm >= 2 ? LBM_ROUND_CTAS : per_sm);
-  RoundArgs ra{rl.h_in, rl.ab_in, rl.h_out, rl.a_out, rl.ab_out, rl.y_out, rl.f_post, rl.f_out,
-               rl.tau, rl.taus, rl.round, rl.h_skip};
-  if (rl.a_from_h) {
-    switch (mode) {
-      case 0: return round_t<0, true>(ra, geo, grid, packed, stw, st);
-      case 1: return round_t<1, true>(ra, geo, grid, packed, stw, st);
-      default: return round_t<2, true>(ra, geo, grid, packed, stw, st);
-    }
-  }
-  switch (mode) {
-    case 0: return round_t<0, false>(ra, geo, grid, packed, stw, st);
-    case 1: return round_t<1, false>(ra, geo, grid, packed, stw, st);
-    default: return round_t<2, false>(ra, geo, grid, packed, stw, st);
-  }
+  return mode == 0 ? round_t<0, true>(round_args(rl), geo, N, per_sm, packed, stw, st)
+                   : round_t<1, true>(round_args(rl), geo, N, per_sm, packed, stw, st);
 }
 
 cudaError_t launch_gnn_encode(const float* f, bool pull, bool b_only, const Shape& s,
@@ -653,7 +674,13 @@ cudaError_t launch_gnn_encode(const float* f, bool pull, bool b_only, const Shap
 
 cudaError_t launch_gnn_round(int mode, const RoundLaunch& rl, const Shape& s,
                              const uint8_t* packed, cudaStream_t st) {
-  return round_any(mode, rl, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx, packed, st);
+  const int64_t N = (int64_t)s.nb * s.ny * s.nx;
+  const GeoStack geo = make_geo_stack(s);
+  if (rl.a_from_h) return round_step(mode, rl, geo, N, packed, st);
+  unsigned* stw = status_word();
+  if (!stw) return cudaErrorInvalidDevice;
+  return mode == 0 ? round_t<0, false>(round_args(rl), geo, N, 2, packed, stw, st)
+                   : round_t<2, false>(round_args(rl), geo, N, 2, packed, stw, st);
 }
 
 // The network forward of the channel (GeoChannel: graph stopped at the
@@ -675,15 +702,12 @@ cudaError_t launch_gnn_forward_channel(const float* f_pre, const Shape& s, float
   if ((e = encode_t<false, false>(f_pre, geo, N, 2, enc::BYTES + 1024, packed, sv.h0, sv.ab0, stw,
                                   st)) != cudaSuccess)
     return e;
-  const int64_t cta_tiles =
-      (N + (int64_t)TILE * LBM_ROUND_GROUPS - 1) / ((int64_t)TILE * LBM_ROUND_GROUPS);
-  const unsigned grid = grid_for(cta_tiles * TILE, LBM_ROUND_CTAS);
   RoundArgs r0{sv.h0, sv.ab0, sv.h1, sv.a0, sv.ab1, nullptr, nullptr, nullptr, 1.0f, nullptr, 0,
                nullptr};
-  if ((e = round_t<0, false>(r0, geo, grid, packed, stw, st)) != cudaSuccess) return e;
+  if ((e = round_t<0, false>(r0, geo, N, 2, packed, stw, st)) != cudaSuccess) return e;
   RoundArgs r1{sv.h1, sv.ab1, sv.h2, sv.a1, nullptr, y, nullptr, nullptr, 1.0f, nullptr, 1,
                nullptr};
-  return round_t<2, false>(r1, geo, grid, packed, stw, st);
+  return round_t<2, false>(r1, geo, N, 2, packed, stw, st);
 }
 
 cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc* lat, int first,
@@ -697,15 +721,9 @@ cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc
   __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(b0 + count * 64);
   __half* b1 = reinterpret_cast<__half*>(h1 + count * 64);
   cudaError_t e;
-  // MLP-only network: the fused step; the kernels below then return at once
-  if ((e = launch_gnn_mlp_step_table(f_in, f_out, lat, first, n, hint, base, count, ps, packed, st,
-                                     per_sm)) != cudaSuccess)
-    return e;
-  // encoder (pull, features, two layers, B = W_b h0): the fused kernel of
-  // gnn_mlp.cu in its encoder mode
-  (void)per_sm;
-  if ((e = launch_gnn_encode_fused_table(f_in, lat, first, n, hint, base, count, ps, packed, h0, b0,
-                                         st)) != cudaSuccess)
+  // the whole step of an MLP-only network, or the encoder (gnn_mlp.cu)
+  if ((e = launch_gnn_encode_fused_table(f_in, f_out, lat, first, n, hint, base, count, ps, packed,
+                                         h0, b0, st)) != cudaSuccess)
     return e;
   RoundLaunch r0;
   r0.h_in = h0;
@@ -715,7 +733,7 @@ cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc
   r0.h_out = h1;
   r0.ab_out = b1;
   r0.round = 0;
-  if ((e = round_any(0, r0, geo, count, packed, st, per_sm)) != cudaSuccess) return e;
+  if ((e = round_step(0, r0, geo, count, packed, st, per_sm)) != cudaSuccess) return e;
   RoundLaunch r1;
   r1.h_in = h1;
   r1.ab_in = b1;
@@ -724,7 +742,7 @@ cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc
   r1.f_post = f_in;
   r1.f_out = f_out;
   r1.round = 1;
-  return round_any(1, r1, geo, count, packed, st, per_sm);
+  return round_step(1, r1, geo, count, packed, st, per_sm);
 }
 
 }  // namespace lbmgnn

@@ -69,27 +69,24 @@ cudaError_t launch_channel_restrict(const float* f_fine, const Shape& fs, float*
 
 // The paper's Fig. 2 network (MLP-only variant) as one fused GNN-LBM step
 // kernel (pull, features, 3 MMAs, heads, Eq. 3, store).  For any other
-// network the kernel writes nothing (and with require_mlp raises ST_BLOB).
+// network the kernel writes nothing and raises ST_BLOB.
 cudaError_t launch_gnn_mlp_step(const float* f_in, float* f_out, const Shape& s, float tau,
-                                const float* taus, const uint8_t* packed, bool require_mlp,
-                                cudaStream_t st);
+                                const float* taus, const uint8_t* packed, cudaStream_t st);
 
 struct LatDesc;
-// The inference encoder of a message-passing network in the fused kernel's
-// design (pull, features, two GELU layers, B = W_b h0; h0 BF16 and B FP16
-// [N][64] in the chunked plane layout); returns at once for the MLP-only
-// network.  The table form takes the nodes [base, base+count) of the lattices
+// The first launch of a GNN-LBM step, for whichever network the image holds:
+// for the MLP-only network its whole step (the round kernels then return at
+// once), else the inference encoder in the same design (pull, features, two
+// GELU layers, B = W_b h0; h0 BF16 and B FP16 [N][64] in the chunked plane
+// layout).  The table form takes the nodes [base, base+count) of the lattices
 // first .. first+n-1 of a device descriptor table.
-cudaError_t launch_gnn_encode_fused(const float* f_in, const Shape& s, const uint8_t* packed,
-                                    __nv_bfloat16* h0, __half* b, cudaStream_t st);
-cudaError_t launch_gnn_encode_fused_table(const float* f_in, const LatDesc* lat, int first, int n,
-                                          const int* hint, int64_t base, int64_t count, int64_t ps,
-                                          const uint8_t* packed, __nv_bfloat16* h0, __half* b,
-                                          cudaStream_t st);
-cudaError_t launch_gnn_mlp_step_table(const float* f_in, float* f_out, const LatDesc* lat,
-                                      int first, int n, const int* hint, int64_t base,
-                                      int64_t count, int64_t ps, const uint8_t* packed,
-                                      cudaStream_t st, int per_sm);
+cudaError_t launch_gnn_encode_fused(const float* f_in, float* f_out, const Shape& s, float tau,
+                                    const float* taus, const uint8_t* packed, __nv_bfloat16* h0,
+                                    __half* b, cudaStream_t st);
+cudaError_t launch_gnn_encode_fused_table(const float* f_in, float* f_out, const LatDesc* lat,
+                                          int first, int n, const int* hint, int64_t base,
+                                          int64_t count, int64_t ps, const uint8_t* packed,
+                                          __nv_bfloat16* h0, __half* b, cudaStream_t st);
 // GNN-LBM step (encoder, 2 rounds, head + Eq. 3) on the lattices first ..
 // first+n-1 of a device descriptor table, whose nodes are [base, base+count)
 // of population buffers with plane stride ps; hint: device int per 128-node

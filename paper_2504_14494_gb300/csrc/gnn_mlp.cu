@@ -157,18 +157,10 @@ __device__ __forceinline__ void gelu_to_tmem(uint32_t lane_d, uint32_t lane_a,
 // round-0 edge term B = W_b h0; h0 (BF16) and B (FP16) go to HBM in the
 // chunked plane layout of the round kernels.
 template <class Geo, bool ENC>
-__global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
-    const float* __restrict__ f_in, float* __restrict__ f_out, Geo geo, float tau0,
-    const float* __restrict__ taus, const uint8_t* __restrict__ packed, bool require_mlp,
-    bool rows, __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ b_out, unsigned* stw) {
-  if (!blob_ok(packed, stw)) return;
-  const int variant = variant_of(reinterpret_cast<const float*>(packed + K::NORM));
-  if (ENC ? (variant & VAR_MLP_ONLY) != 0 : !(variant & VAR_MLP_ONLY)) {
-    // the MLP-only network is stepped by the MLP mode alone; message-passing
-    // networks by the encoder mode and the round kernels
-    if (!ENC && require_mlp && threadIdx.x == 0) raise_status(stw, ST_BLOB);
-    return;
-  }
+__device__ __forceinline__ void mlp_or_encode(
+    const float* __restrict__ f_in, float* __restrict__ f_out, const Geo& geo, float tau0,
+    const float* __restrict__ taus, const uint8_t* __restrict__ packed, int variant, bool rows,
+    __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ b_out, unsigned* stw) {
   extern __shared__ uint8_t smem_raw[];
   // aligned through an integer: the staged populations are then read with
   // generic loads, measured faster here than shared-memory loads (the other
@@ -183,8 +175,11 @@ __global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
   const int64_t N = geo.count();
   const int64_t base = geo.base(), ps = geo.ps();
   const int64_t ntiles = (N + TILE - 1) / TILE;
-  const int64_t first = (int64_t)blockIdx.x * mlp::NG + grp,
-                stride = (int64_t)gridDim.x * mlp::NG;
+  // tiles: the groups of a CTA take neighbouring ones, or, where not every
+  // group of the grid has one, every SM takes one before any takes a second
+  const int64_t stride = (int64_t)gridDim.x * mlp::NG;
+  const int64_t first = ntiles < stride ? (int64_t)grp * gridDim.x + blockIdx.x
+                                        : (int64_t)blockIdx.x * mlp::NG + grp;
 
   // The pulled populations of tile `tile` -> stage st (cp.async), and each
   // node's relaxation time.  rows (a stack whose rows are whole tiles,
@@ -501,59 +496,68 @@ __global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
   if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, mlp::TM_COLS);
 }
 
-template <class Geo, bool ENC = false>
+// STEP = false: the step of the MLP-only network (another one is refused).
+// STEP = true: the first launch of a GNN-LBM step, whichever network the image
+// holds: the whole step of an MLP-only one, the encoder of any other.
+template <class Geo, bool STEP>
+__global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
+    const float* __restrict__ f_in, float* __restrict__ f_out, Geo geo, float tau0,
+    const float* __restrict__ taus, const uint8_t* __restrict__ packed, bool rows,
+    __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ b_out, unsigned* stw) {
+  dep_sync();  // (the first kernel of a call: no wait; the next one may set up)
+  if (!blob_ok(packed, stw)) return;
+  const int variant = variant_of(reinterpret_cast<const float*>(packed + K::NORM));
+  if (variant & VAR_MLP_ONLY)
+    mlp_or_encode<Geo, false>(f_in, f_out, geo, tau0, taus, packed, variant, rows, nullptr, nullptr,
+                              stw);
+  else if constexpr (STEP)
+    mlp_or_encode<Geo, true>(f_in, nullptr, geo, 1.0f, nullptr, packed, 0, rows, h0_out, b_out, stw);
+  else if (threadIdx.x == 0)
+    raise_status(stw, ST_BLOB);
+}
+
+template <class Geo, bool STEP>
 static cudaError_t mlp_step(const float* f_in, float* f_out, const Geo& geo, int64_t N, float tau,
-                            const float* taus, const uint8_t* packed, bool require_mlp, bool rows,
-                            cudaStream_t st, __nv_bfloat16* h0 = nullptr, __half* b = nullptr) {
+                            const float* taus, const uint8_t* packed, bool rows, cudaStream_t st,
+                            __nv_bfloat16* h0 = nullptr, __half* b = nullptr) {
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   if (N <= 0) return cudaSuccess;
   const uint32_t bytes = mlp::BYTES + 1024;
   cudaError_t e;
-  if ((e = set_smem(gnn_mlp_step_kernel<Geo, ENC>, bytes)) != cudaSuccess) return e;
+  if ((e = set_smem(gnn_mlp_step_kernel<Geo, STEP>, bytes)) != cudaSuccess) return e;
   // one CTA (NG tile groups) per SM, fewer for small lattices
   const int64_t ntiles = (N + TILE - 1) / TILE;
-  const int64_t want = (ntiles + mlp::NG - 1) / mlp::NG;
-  const unsigned grid = (unsigned)(want < num_sms() ? want : num_sms());
-  gnn_mlp_step_kernel<Geo, ENC><<<grid, 128 * mlp::NG, bytes, st>>>(
-      f_in, f_out, geo, tau, taus, packed, require_mlp, rows, h0, b, stw);
+  const unsigned grid = (unsigned)(ntiles < num_sms() ? ntiles : num_sms());
+  gnn_mlp_step_kernel<Geo, STEP><<<grid, 128 * mlp::NG, bytes, st>>>(
+      f_in, f_out, geo, tau, taus, packed, rows, h0, b, stw);
   return cudaGetLastError();
 }
 
+// row runs: every tile inside one lattice row, 16-byte aligned population planes
+static bool row_runs(const float* f_in, const Shape& s) {
+  return s.nx % TILE == 0 && s.ps % 4 == 0 && (reinterpret_cast<uintptr_t>(f_in) & 15) == 0;
+}
+
 cudaError_t launch_gnn_mlp_step(const float* f_in, float* f_out, const Shape& s, float tau,
-                                const float* taus, const uint8_t* packed, bool require_mlp,
-                                cudaStream_t st) {
-  // row runs: every tile inside one lattice row, 16-byte aligned population planes
-  const bool rows = s.nx % TILE == 0 && s.ps % 4 == 0 &&
-                    (reinterpret_cast<uintptr_t>(f_in) & 15) == 0;
-  return mlp_step(f_in, f_out, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx, tau, taus, packed,
-                  require_mlp, rows, st);
+                                const float* taus, const uint8_t* packed, cudaStream_t st) {
+  return mlp_step<GeoStack, false>(f_in, f_out, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx,
+                                   tau, taus, packed, row_runs(f_in, s), st);
 }
 
-cudaError_t launch_gnn_encode_fused(const float* f_in, const Shape& s, const uint8_t* packed,
-                                    __nv_bfloat16* h0, __half* b, cudaStream_t st) {
-  const bool rows = s.nx % TILE == 0 && s.ps % 4 == 0 &&
-                    (reinterpret_cast<uintptr_t>(f_in) & 15) == 0;
-  return mlp_step<GeoStack, true>(f_in, nullptr, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx,
-                                  1.0f, nullptr, packed, false, rows, st, h0, b);
+cudaError_t launch_gnn_encode_fused(const float* f_in, float* f_out, const Shape& s, float tau,
+                                    const float* taus, const uint8_t* packed, __nv_bfloat16* h0,
+                                    __half* b, cudaStream_t st) {
+  return mlp_step<GeoStack, true>(f_in, f_out, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx,
+                                  tau, taus, packed, row_runs(f_in, s), st, h0, b);
 }
 
-cudaError_t launch_gnn_encode_fused_table(const float* f_in, const LatDesc* lat, int first, int n,
-                                          const int* hint, int64_t base, int64_t count, int64_t ps,
-                                          const uint8_t* packed, __nv_bfloat16* h0, __half* b,
-                                          cudaStream_t st) {
+cudaError_t launch_gnn_encode_fused_table(const float* f_in, float* f_out, const LatDesc* lat,
+                                          int first, int n, const int* hint, int64_t base,
+                                          int64_t count, int64_t ps, const uint8_t* packed,
+                                          __nv_bfloat16* h0, __half* b, cudaStream_t st) {
   const GeoTable geo{lat, first, n, base, count, ps, hint};
-  return mlp_step<GeoTable, true>(f_in, nullptr, geo, count, 0.0f, nullptr, packed, false, false,
-                                  st, h0, b);
-}
-
-cudaError_t launch_gnn_mlp_step_table(const float* f_in, float* f_out, const LatDesc* lat,
-                                      int first, int n, const int* hint, int64_t base,
-                                      int64_t count, int64_t ps, const uint8_t* packed,
-                                      cudaStream_t st, int per_sm) {
-  const GeoTable geo{lat, first, n, base, count, ps, hint};
-  (void)per_sm;  // one CTA of LBM_MLP_GROUPS tile groups per SM, whatever the batch plan chose
-  return mlp_step(f_in, f_out, geo, count, 0.0f, nullptr, packed, false, false, st);
+  return mlp_step<GeoTable, true>(f_in, f_out, geo, count, 0.0f, nullptr, packed, false, st, h0, b);
 }
 
 }  // namespace lbmgnn

@@ -6,6 +6,28 @@
 
 namespace lbmgnn {
 
+// Launch that, with `early`, may start before the preceding kernel on `st` has
+// completed; the kernel waits for it in dep_sync() (common.cuh).  Early only
+// while the kernels of a call need one CTA per SM: the shared-memory split of
+// an SM cannot change under a running CTA, so the CTAs of a kernel that wants
+// two per SM, started early, ran one per SM (1024^2 GNN-LBM step 599 us
+// against 546; 64^2, one CTA per SM: 23 against 35).
+template <typename... Params, typename... Args>
+inline cudaError_t launch_after(bool early, void (*kern)(Params...), unsigned grid, unsigned block,
+                                size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 cudaError_t launch_bgk_step(const float* fin, float* fout, const Shape& s, float tau,
                             const float* taus, double* totals, cudaStream_t st);
 // The step restricted to lattice rows row0 .. row1-1 (of the nb*ny rows).
