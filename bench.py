@@ -563,7 +563,7 @@ def gnn_bench(args, L, dev, stream, side=GNN_SIDE, only=False, theta=None, label
     return {"workload": f"tgv_gnn_{n}x{n}", "re": GNN_RE, "tau": round(tau, 5), "u0": U0,
             "roofline": None if mlp_only else {
                 "bound": "alu",
-                "kernel": "lbm_step_gnn (fused encoder gnn_mlp_step_kernel<ENC> + 2 x gnn_round_kernel)",
+                "kernel": "lbm_step_gnn (fused encoder gnn_step_first_kernel + 2 x gnn_round_kernel)",
                 "peak_basis": f"{GELU_PER_CLK_SM:.2f} edge GELUs/clock/SM x {_sm_count(dev)} SMs "
                               f"x {_max_sm_hz(dev) / 1e6:.0f} MHz (measured issue rate of the "
                               f"message sequence, MUFU tanh bound; microbench/fp16_rate.cu)",

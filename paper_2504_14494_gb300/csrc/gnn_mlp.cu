@@ -175,11 +175,12 @@ __device__ __forceinline__ void mlp_or_encode(
   const int64_t N = geo.count();
   const int64_t base = geo.base(), ps = geo.ps();
   const int64_t ntiles = (N + TILE - 1) / TILE;
-  // tiles: the groups of a CTA take neighbouring ones, or, where not every
-  // group of the grid has one, every SM takes one before any takes a second
+  // tiles: the groups of a CTA take neighbouring ones, or, in the encoder where
+  // not every group of the grid has one, every SM takes one before any takes a
+  // second
   const int64_t stride = (int64_t)gridDim.x * mlp::NG;
-  const int64_t first = ntiles < stride ? (int64_t)grp * gridDim.x + blockIdx.x
-                                        : (int64_t)blockIdx.x * mlp::NG + grp;
+  const int64_t first = ENC && ntiles < stride ? (int64_t)grp * gridDim.x + blockIdx.x
+                                               : (int64_t)blockIdx.x * mlp::NG + grp;
 
   // The pulled populations of tile `tile` -> stage st (cp.async), and each
   // node's relaxation time.  rows (a stack whose rows are whole tiles,
@@ -496,41 +497,69 @@ __device__ __forceinline__ void mlp_or_encode(
   if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, mlp::TM_COLS);
 }
 
-// STEP = false: the step of the MLP-only network (another one is refused).
-// STEP = true: the first launch of a GNN-LBM step, whichever network the image
-// holds: the whole step of an MLP-only one, the encoder of any other.
-template <class Geo, bool STEP>
-__global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
-    const float* __restrict__ f_in, float* __restrict__ f_out, Geo geo, float tau0,
-    const float* __restrict__ taus, const uint8_t* __restrict__ packed, bool rows,
-    __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ b_out, unsigned* stw) {
-  dep_sync();  // (the first kernel of a call: no wait; the next one may set up)
-  if (!blob_ok(packed, stw)) return;
-  const int variant = variant_of(reinterpret_cast<const float*>(packed + K::NORM));
-  if (variant & VAR_MLP_ONLY)
-    mlp_or_encode<Geo, false>(f_in, f_out, geo, tau0, taus, packed, variant, rows, nullptr, nullptr,
-                              stw);
-  else if constexpr (STEP)
-    mlp_or_encode<Geo, true>(f_in, nullptr, geo, 1.0f, nullptr, packed, 0, rows, h0_out, b_out, stw);
-  else if (threadIdx.x == 0)
-    raise_status(stw, ST_BLOB);
+template <class Geo>
+struct MlpArgs {
+  const float* f_in;
+  float* f_out;
+  Geo geo;
+  float tau0;
+  const float* taus;
+  const uint8_t* packed;
+  bool rows;
+  __nv_bfloat16* h0;
+  __half* b;
+  unsigned* stw;
+};
+// Out of line in the kernel that holds both networks: inlined, its registers
+// cost the encoder 3 us at 1024^2.
+template <class Geo>
+__device__ __noinline__ void mlp_only_step(const MlpArgs<Geo>* a, int variant) {
+  mlp_or_encode<Geo, false>(a->f_in, a->f_out, a->geo, a->tau0, a->taus, a->packed, variant,
+                            a->rows, nullptr, nullptr, a->stw);
 }
 
-template <class Geo, bool STEP>
-static cudaError_t mlp_step(const float* f_in, float* f_out, const Geo& geo, int64_t N, float tau,
-                            const float* taus, const uint8_t* packed, bool rows, cudaStream_t st,
-                            __nv_bfloat16* h0 = nullptr, __half* b = nullptr) {
-  unsigned* stw = status_word();
-  if (!stw) return cudaErrorInvalidDevice;
+// The step of the MLP-only network; another one is refused.
+template <class Geo>
+__global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
+    const float* __restrict__ f_in, float* __restrict__ f_out, Geo geo, float tau0,
+    const float* __restrict__ taus, const uint8_t* __restrict__ packed, bool rows, unsigned* stw) {
+  if (!blob_ok(packed, stw)) return;
+  const int variant = variant_of(reinterpret_cast<const float*>(packed + K::NORM));
+  if (!(variant & VAR_MLP_ONLY)) {
+    if (threadIdx.x == 0) raise_status(stw, ST_BLOB);
+    return;
+  }
+  mlp_or_encode<Geo, false>(f_in, f_out, geo, tau0, taus, packed, variant, rows, nullptr, nullptr,
+                            stw);
+}
+
+// The first launch of a GNN-LBM step, whichever network the image holds: the
+// whole step of an MLP-only one, the encoder of any other.
+template <class Geo>
+__global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1)
+    gnn_step_first_kernel(const __grid_constant__ MlpArgs<Geo> a) {
+  dep_sync();  // (the first kernel of a call: the next one may set up)
+  if (!blob_ok(a.packed, a.stw)) return;
+  const int variant = variant_of(reinterpret_cast<const float*>(a.packed + K::NORM));
+  if (variant & VAR_MLP_ONLY)
+    mlp_only_step<Geo>(&a, variant);
+  else
+    mlp_or_encode<Geo, true>(a.f_in, nullptr, a.geo, 1.0f, nullptr, a.packed, 0, a.rows, a.h0, a.b,
+                             a.stw);
+}
+
+template <class Geo>
+static cudaError_t step_first(MlpArgs<Geo> a, int64_t N, cudaStream_t st) {
+  a.stw = status_word();
+  if (!a.stw) return cudaErrorInvalidDevice;
   if (N <= 0) return cudaSuccess;
   const uint32_t bytes = mlp::BYTES + 1024;
   cudaError_t e;
-  if ((e = set_smem(gnn_mlp_step_kernel<Geo, STEP>, bytes)) != cudaSuccess) return e;
-  // one CTA (NG tile groups) per SM, fewer for small lattices
+  if ((e = set_smem(gnn_step_first_kernel<Geo>, bytes)) != cudaSuccess) return e;
+  // one CTA (NG tile groups) per SM
   const int64_t ntiles = (N + TILE - 1) / TILE;
   const unsigned grid = (unsigned)(ntiles < num_sms() ? ntiles : num_sms());
-  gnn_mlp_step_kernel<Geo, STEP><<<grid, 128 * mlp::NG, bytes, st>>>(
-      f_in, f_out, geo, tau, taus, packed, rows, h0, b, stw);
+  gnn_step_first_kernel<Geo><<<grid, 128 * mlp::NG, bytes, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -541,23 +570,35 @@ static bool row_runs(const float* f_in, const Shape& s) {
 
 cudaError_t launch_gnn_mlp_step(const float* f_in, float* f_out, const Shape& s, float tau,
                                 const float* taus, const uint8_t* packed, cudaStream_t st) {
-  return mlp_step<GeoStack, false>(f_in, f_out, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx,
-                                   tau, taus, packed, row_runs(f_in, s), st);
+  unsigned* stw = status_word();
+  if (!stw) return cudaErrorInvalidDevice;
+  const uint32_t bytes = mlp::BYTES + 1024;
+  cudaError_t e;
+  if ((e = set_smem(gnn_mlp_step_kernel<GeoStack>, bytes)) != cudaSuccess) return e;
+  // one CTA (NG tile groups) per SM, fewer for small lattices
+  const int64_t ntiles = ((int64_t)s.nb * s.ny * s.nx + TILE - 1) / TILE;
+  const int64_t want = (ntiles + mlp::NG - 1) / mlp::NG;
+  const unsigned grid = (unsigned)(want < num_sms() ? want : num_sms());
+  gnn_mlp_step_kernel<GeoStack><<<grid, 128 * mlp::NG, bytes, st>>>(
+      f_in, f_out, make_geo_stack(s), tau, taus, packed, row_runs(f_in, s), stw);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_gnn_encode_fused(const float* f_in, float* f_out, const Shape& s, float tau,
                                     const float* taus, const uint8_t* packed, __nv_bfloat16* h0,
                                     __half* b, cudaStream_t st) {
-  return mlp_step<GeoStack, true>(f_in, f_out, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx,
-                                  tau, taus, packed, row_runs(f_in, s), st, h0, b);
+  return step_first(MlpArgs<GeoStack>{f_in, f_out, make_geo_stack(s), tau, taus, packed,
+                                      row_runs(f_in, s), h0, b, nullptr},
+                    (int64_t)s.nb * s.ny * s.nx, st);
 }
 
 cudaError_t launch_gnn_encode_fused_table(const float* f_in, float* f_out, const LatDesc* lat,
                                           int first, int n, const int* hint, int64_t base,
                                           int64_t count, int64_t ps, const uint8_t* packed,
                                           __nv_bfloat16* h0, __half* b, cudaStream_t st) {
-  const GeoTable geo{lat, first, n, base, count, ps, hint};
-  return mlp_step<GeoTable, true>(f_in, f_out, geo, count, 0.0f, nullptr, packed, false, st, h0, b);
+  return step_first(MlpArgs<GeoTable>{f_in, f_out, GeoTable{lat, first, n, base, count, ps, hint},
+                                      0.0f, nullptr, packed, false, h0, b, nullptr},
+                    count, st);
 }
 
 }  // namespace lbmgnn
