@@ -17,6 +17,15 @@ __device__ __forceinline__ float2 rcp2_mid(float2 x) {
   return __ffma2_rn(r, e, r);
 }
 
+// The same for one value, any x.
+__device__ __forceinline__ float rcp1(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  r = __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
+  if (!(x >= 0x1p-90f && x <= 0x1p90f)) r = 1.0f / x;
+  return r;
+}
+
 // bgk_collide() of 2 NP nodes in packed FP32 pairs (one instruction for two
 // nodes), nomega = -1/tau: the same roundings in the same order as the
 // compiler makes of bgk_collide (products contracted into the following
@@ -71,13 +80,41 @@ __device__ __forceinline__ void bgk_collide_pairs(float2 (&f)[Q][NP], float2 nom
   }
 }
 
+// bgk_collide() of one node, the same way as bgk_collide_pairs.
+__device__ __forceinline__ void bgk_collide_one(float (&f)[Q], float omega) {
+  const float rho = __fadd_rn(
+      __fadd_rn(__fadd_rn(f[0], __fadd_rn(f[1], f[3])), __fadd_rn(f[2], f[4])),
+      __fadd_rn(__fadd_rn(f[5], f[7]), __fadd_rn(f[6], f[8])));
+  const float inv = rcp1(rho);
+  const float d57 = __fsub_rn(f[5], f[7]), d86 = __fsub_rn(f[8], f[6]);
+  const float ux = __fmul_rn(__fadd_rn(__fadd_rn(__fsub_rn(f[1], f[3]), d57), d86), inv);
+  const float uy = __fmul_rn(__fsub_rn(__fadd_rn(__fsub_rn(f[2], f[4]), d57), d86), inv);
+  const float poison = __fmaf_rn(0.0f, ux, __fmul_rn(0.0f, uy));
+  const float usq = __fadd_rn(__fmaf_rn(ux, ux, __fmul_rn(uy, uy)), poison);
+  auto relax = [&](int q, float t, float nwr) {
+    t = __fmaf_rn(-1.5f, usq, t);
+    f[q] = __fmaf_rn(-omega, __fmaf_rn(nwr, t, f[q]), f[q]);
+  };
+  auto both = [&](int q, int o, float eu, float nwr) {
+    const float a = __fmul_rn(4.5f, eu);
+    relax(q, __fmaf_rn(a, eu, __fmaf_rn(3.0f, eu, 1.0f)), nwr);
+    relax(o, __fmaf_rn(a, eu, __fmaf_rn(-3.0f, eu, 1.0f)), nwr);
+  };
+  const float w1 = __fmul_rn(-wq(1), rho), w5 = __fmul_rn(-wq(5), rho);
+  relax(0, 1.0f, __fmul_rn(-wq(0), rho));
+  both(1, 3, ux, w1);
+  both(2, 4, uy, w1);
+  both(5, 7, __fadd_rn(ux, uy), w5);
+  both(6, 8, __fsub_rn(uy, ux), w5);
+}
+
 // f_i - (f_i - f_i^eq(rho, u))/t + (1 - 1/(2t)) w_i [3 (e_i - u) + 9 (e_i.u) e_i].(gx, 0)
 // with u the force-corrected velocity; t is tau (BGK) or tau tau_adj (Eq. 3).
 __device__ __forceinline__ void channel_relax(float (&f)[Q], float t, float gx) {
   const float rho = ((f[0] + (f[1] + f[3])) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]));
   const float jx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
   const float jy = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-  const float inv = 1.0f / rho;
+  const float inv = rcp1(rho);
   const Moments m{rho, (jx + 0.5f * gx) * inv, jy * inv};
   const float usq15 = 1.5f * (m.ux * m.ux + m.uy * m.uy);
   const float omega = 1.0f / t, pre = 1.0f - 0.5f * omega;

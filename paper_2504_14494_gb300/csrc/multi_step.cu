@@ -10,9 +10,9 @@
 // by the latency of one step: one thread-block cluster (1..8 CTAs) per lattice
 // holds the whole lattice in shared memory (two buffers) for all steps of the
 // call; per step a pull from shared memory, the collision, a store to the
-// other buffer (edge rows also to the neighbouring CTAs' halo rows through
-// distributed shared memory) and one cluster barrier.  64^2: 0.75 us a step
-// (4.1 with one launch a step); a 4 x 32 channel: 0.33 (4.1).
+// other buffer, edge rows also to the neighbouring CTAs' halo rows through
+// distributed shared memory.  64^2: 0.54 us a step (4.1 with one launch a
+// step); a 4 x 32 channel, in one CTA: 0.23 (4.1).
 //
 // temporal_steps_kernel -- for larger lattices, which are bound by memory
 // traffic (72 bytes per node and step): T = 2..4 steps per pass over memory.
@@ -35,6 +35,7 @@
 
 #include "collide.cuh"
 #include "launch.h"
+#include "umma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -58,7 +59,16 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
 
 // ---------------------------------------------------------------------------
 // Resident form.  CTA r of the cluster holds rows r R .. min(ny, (r + 1) R) - 1
-// of lattice b as local rows 1..; local rows 0 and rows + 1 are the halo.
+// of lattice b as local rows 1..; local rows 0 and rows + 1 are the halo
+// (unused by a CTA that holds the whole lattice).
+//
+// Between two steps the CTAs of a cluster exchange their edge rows: each edge
+// node's three outgoing populations go to the neighbour's halo row by st.async,
+// which counts their bytes on an mbarrier there; the threads of the edge rows
+// wait for the halo's bytes, the others only for their own CTA.  (A cluster
+// barrier per step in its place: 0.75 us a step at 64^2.)  There is one
+// mbarrier per buffer: a CTA cannot start step n + 2 before its neighbours have
+// sent step n + 1, so a neighbour is at most one step ahead.
 struct ResidentArgs {
   const float* fin;
   float* fout;
@@ -70,21 +80,50 @@ struct ResidentArgs {
   int rows;    // R: rows per CTA
 };
 
-// KN: nodes per thread.  CH: the channel (bounce-back walls, force gx).
-template <bool CH, int KN>
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_async(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
+                   addr),
+               "r"(__float_as_uint(v)), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void expect_bytes(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+
+// KN: nodes per thread.  CH: the channel (bounce-back walls, force gx).  ONE:
+// the whole lattice in one CTA.
+template <bool CH, int KN, bool ONE>
 __global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, unsigned* stw) {
   extern __shared__ float sm[];
+  __shared__ uint64_t bar[2];
   cg::cluster_group cl = cg::this_cluster();
-  const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
+  const int C = ONE ? 1 : (int)cl.num_blocks(), r = ONE ? 0 : (int)cl.block_rank();
   const int nx = a.s.nx, ny = a.s.ny;
   const int64_t b = blockIdx.x / C, lat = b * ny * nx;
   const int ya = r * a.rows, rows = min(ny - ya, a.rows);
   const int pitch = (a.rows + 2) * nx;  // one plane
-  float *cur = sm, *nxt = sm + Q * pitch;
+  const uint32_t halo_bytes = 2u * 3u * 4u * (uint32_t)nx;
+  if constexpr (!ONE) {
+    if (threadIdx.x == 0) {
+      mbar_init(&bar[0], 1);
+      mbar_init(&bar[1], 1);
+      expect_bytes(&bar[0], halo_bytes);
+      expect_bytes(&bar[1], halo_bytes);
+    }
+  }
   // the neighbours (periodic): the CTA holding row ya - 1 and the one holding
   // row ya + rows, and the local index of the halo row this CTA fills there
   const int up = r == 0 ? C - 1 : r - 1, dn = r == C - 1 ? 0 : r + 1;
   const int up_rows = min(ny - up * a.rows, a.rows);
+  const uint32_t up_sm = map_rank(smem_u32(sm), up), dn_sm = map_rank(smem_u32(sm), dn);
+  const uint32_t up_bar = map_rank(smem_u32(bar), up), dn_bar = map_rank(smem_u32(bar), dn);
   const float* fin = a.fin + lat;
   // own rows and both halo rows
   for (int i = threadIdx.x; i < (rows + 2) * nx; i += blockDim.x) {
@@ -93,103 +132,125 @@ __global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, un
     y = y < 0 ? ny - 1 : (y >= ny ? 0 : y);
 #pragma unroll
     for (int q = 0; q < Q; ++q)
-      cur[q * pitch + i] = __ldg(
+      sm[q * pitch + i] = __ldg(
           fin + q * a.s.ps + checked((int64_t)y * nx + x, 0, (int64_t)ny * nx, stw));
   }
-  // this thread's nodes: offset of (local row, 0), x -+ 1 with wrap
-  int row0[KN], xc[KN], xl[KN], xr[KN], ly[KN];
+  // this thread's nodes: own offset, and the sources of the nine populations
+  int own[KN], src[KN][Q];
+  bool first_row[KN], last_row[KN];
 #pragma unroll
   for (int k = 0; k < KN; ++k) {
     const int i = threadIdx.x + k * blockDim.x;
-    ly[k] = i < rows * nx ? i / nx : -1;
-    xc[k] = ly[k] < 0 ? 0 : i - ly[k] * nx;
-    row0[k] = (max(ly[k], 0) + 1) * nx;
-    xl[k] = xc[k] == 0 ? nx - 1 : xc[k] - 1;
-    xr[k] = xc[k] == nx - 1 ? 0 : xc[k] + 1;
+    const int ly = i < rows * nx ? i / nx : -1;
+    const int x = ly < 0 ? 0 : i - ly * nx, y = ya + ly;
+    first_row[k] = ly == 0;
+    last_row[k] = ly == rows - 1;
+    own[k] = ly < 0 ? -1 : (ly + 1) * nx + x;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      int xs = x - ex(q), ls = ly + 1 - ey(q);
+      xs = xs < 0 ? nx - 1 : (xs >= nx ? 0 : xs);
+      if (ONE && !CH) ls = ls < 1 ? rows : (ls > rows ? 1 : ls);
+      src[k][q] = q * pitch + ls * nx + xs;
+      if (CH && (y - ey(q) < 0 || y - ey(q) >= ny)) src[k][q] = opp(q) * pitch + own[k];  // bounce-back
+      if (ly < 0) src[k][q] = 0;
+    }
   }
   const float tau = a.taus ? __ldg(a.taus + b) : a.tau;
   const float omega = 1.0f / tau;
-  float* up_sm = cl.map_shared_rank(sm, up);
-  float* dn_sm = cl.map_shared_rank(sm, dn);
-  if (C == 1) __syncthreads(); else cl.sync();
+  if constexpr (ONE) __syncthreads(); else cl.sync();
 
+  int cur = 0, nxt = Q * pitch;
   for (int step = 0; step < a.nsteps; ++step) {
-    const int nxt_off = (int)(nxt - sm);
     const bool last = step == a.nsteps - 1;
+    bool lost = false;  // a neighbour's rows never came
 #pragma unroll
     for (int k = 0; k < KN; ++k) {
-      if (ly[k] < 0) continue;
-      float f[Q];
-      const bool lo = CH && ya + ly[k] == 0, hi = CH && ya + ly[k] == ny - 1;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int xs = ex(q) == 0 ? xc[k] : (ex(q) > 0 ? xl[k] : xr[k]);
-        int o = q * pitch + row0[k] - ey(q) * nx + xs;
-        if (ey(q) > 0 && lo) o = opp(q) * pitch + row0[k] + xc[k];  // halfway bounce-back
-        if (ey(q) < 0 && hi) o = opp(q) * pitch + row0[k] + xc[k];
-        f[q] = cur[o];
+      if (own[k] < 0) continue;
+      if constexpr (!ONE) {
+        // the halo of this step's buffer (step 0: loaded above)
+        if (step > 0 && (first_row[k] || last_row[k])) {
+          const int h = step & 1;  // filled during step - 1
+          if (!mbar_wait(&bar[h], ((step - 1) >> 1) & 1)) lost = true;
+          if (k == 0 && threadIdx.x == 0) expect_bytes(&bar[h], halo_bytes);  // for step + 2
+        }
       }
-      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide(f, omega);
+      float f[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) f[q] = sm[cur + src[k][q]];
+      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide_one(f, omega);
       if (last) {
-        float* o = a.fout + lat + (int64_t)(ya + ly[k]) * nx + xc[k];
+        float* o = a.fout + lat + (int64_t)(ya - 1) * nx + own[k];
 #pragma unroll
         for (int q = 0; q < Q; ++q) o[q * a.s.ps] = f[q];
       } else {
-        const int o = row0[k] + xc[k];
+        float* o = sm + nxt + own[k];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) nxt[q * pitch + o] = f[q];
-        // the rows the neighbours pull across the cut (the channel's walls
-        // need none, and nothing reads what is stored for them)
-        if (ly[k] == 0) {  // e_y = -1: below the last row of `up`
-          float* h = up_sm + nxt_off + (up_rows + 1) * nx + xc[k];
-          h[4 * pitch] = f[4], h[7 * pitch] = f[7], h[8 * pitch] = f[8];
-        }
-        if (ly[k] == rows - 1) {  // e_y = +1: above the first row of `dn`
-          float* h = dn_sm + nxt_off + xc[k];
-          h[2 * pitch] = f[2], h[5 * pitch] = f[5], h[6 * pitch] = f[6];
+        for (int q = 0; q < Q; ++q) o[q * pitch] = f[q];
+        if constexpr (!ONE) {
+          // the rows the neighbours pull across the cut (across the channel's
+          // walls too, where nothing reads them: the byte counts stay alike)
+          const uint32_t h = 8u * ((step + 1) & 1);
+          if (first_row[k]) {  // e_y = -1: below the last row of `up`
+            const uint32_t o4 = up_sm + 4u * (nxt + own[k] + up_rows * nx);
+            st_async(o4 + 16u * pitch, f[4], up_bar + h);
+            st_async(o4 + 28u * pitch, f[7], up_bar + h);
+            st_async(o4 + 32u * pitch, f[8], up_bar + h);
+          }
+          if (last_row[k]) {  // e_y = +1: above the first row of `dn`
+            const uint32_t o4 = dn_sm + 4u * (nxt + own[k] - rows * nx);
+            st_async(o4 + 8u * pitch, f[2], dn_bar + h);
+            st_async(o4 + 20u * pitch, f[5], dn_bar + h);
+            st_async(o4 + 24u * pitch, f[6], dn_bar + h);
+          }
         }
       }
     }
-    if (C == 1) __syncthreads(); else cl.sync();
-    float* t = cur;
+    if constexpr (ONE) {
+      __syncthreads();
+    } else if (__syncthreads_or(lost)) {
+      if (threadIdx.x == 0) raise_status(stw, ST_TIMEOUT);
+      break;
+    }
+    const int t = cur;
     cur = nxt;
     nxt = t;
   }
+  // no CTA leaves while a neighbour may still reach into its shared memory
+  if constexpr (!ONE) cl.sync();
 }
 
-constexpr int SMEM_MAX = 227 * 1024;
+constexpr int SMEM_MAX = 227 * 1024 - 64;  // (64: the mbarriers)
 
 uint32_t resident_smem(int rows, int nx) { return 2u * Q * (uint32_t)(rows + 2) * nx * 4u; }
 
-// Cluster size and rows per CTA, or C = 0 when the lattice does not fit.
+// Cluster size and rows per CTA, or C = 0 when the lattice does not fit.  Up to
+// 512 nodes one CTA without an exchange is faster than several (8 x 32 channel:
+// 0.26 us a step against 0.44), above that the largest cluster.
 struct ResidentPlan {
   int C, rows, threads, kn;
 };
 ResidentPlan plan_resident(const Shape& s) {
-  ResidentPlan best{0, 0, 0, 0};
-  if ((int64_t)s.nx * s.ny > 8 * 3072) return best;
-  for (int C = 8; C >= 1; C >>= 1) {
+  const int64_t all = (int64_t)s.nx * s.ny;
+  if (all > 8 * 3072) return {0, 0, 0, 0};
+  for (int C = all <= 512 ? 1 : 8; C >= 1; C >>= 1) {
     if (C > s.ny) continue;
     const int rows = (s.ny + C - 1) / C;
     if ((int64_t)rows * (C - 1) >= s.ny) continue;  // a CTA without rows
-    if (resident_smem(rows, s.nx) > (uint32_t)SMEM_MAX) break;
     const int nodes = rows * s.nx;
     const int kn = (nodes + 1023) / 1024;
-    if (kn > 3) break;
-    const int threads = ((nodes + kn - 1) / kn + 31) / 32 * 32;
-    // keep the largest cluster unless its CTAs would be less than 4 warps
-    if (best.C && best.threads * best.kn >= 128) break;
-    best = {C, rows, threads, kn};
+    if (kn > 3 || resident_smem(rows, s.nx) > (uint32_t)SMEM_MAX) break;
+    return {C, rows, ((nodes + kn - 1) / kn + 31) / 32 * 32, kn};
   }
-  return best;
+  return {0, 0, 0, 0};
 }
 
-template <bool CH, int KN>
+template <bool CH, int KN, bool ONE>
 cudaError_t resident_t(const ResidentArgs& a, const ResidentPlan& p, cudaStream_t st) {
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   const uint32_t bytes = resident_smem(p.rows, a.s.nx);
-  auto* kern = resident_steps_kernel<CH, KN>;
+  auto* kern = resident_steps_kernel<CH, KN, ONE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -208,10 +269,17 @@ cudaError_t resident_t(const ResidentArgs& a, const ResidentPlan& p, cudaStream_
 
 template <bool CH>
 cudaError_t resident(const ResidentArgs& a, const ResidentPlan& p, cudaStream_t st) {
+  if (p.C == 1) {
+    switch (p.kn) {
+      case 1: return resident_t<CH, 1, true>(a, p, st);
+      case 2: return resident_t<CH, 2, true>(a, p, st);
+      default: return resident_t<CH, 3, true>(a, p, st);
+    }
+  }
   switch (p.kn) {
-    case 1: return resident_t<CH, 1>(a, p, st);
-    case 2: return resident_t<CH, 2>(a, p, st);
-    default: return resident_t<CH, 3>(a, p, st);
+    case 1: return resident_t<CH, 1, false>(a, p, st);
+    case 2: return resident_t<CH, 2, false>(a, p, st);
+    default: return resident_t<CH, 3, false>(a, p, st);
   }
 }
 
@@ -429,12 +497,15 @@ double single_us(const Shape& s) {
 }
 
 // `nsteps` steps of the resident form: 4 for the launch; per wave of clusters
-// (about 16 of 8 CTAs run at once) 4 to load and store; per step 0.45 for the
-// cluster barrier and the chain of one node and 0.75e-3 per node of a CTA.
+// (about 16 of 8 CTAs run at once) 4 to load and store; per step the chain of
+// one node and the exchange, and the nodes of a CTA (more than one per thread
+// at half the rate).
 double resident_us(const Shape& s, const ResidentPlan& p, int nsteps) {
   const int at_once = 128 / p.C;
   const double waves = (double)((s.nb + at_once - 1) / at_once);
-  return 4.0 + waves * (4.0 + nsteps * (0.45 + 0.75e-3 * p.rows * s.nx));
+  const double nodes = (double)p.rows * s.nx;
+  const double step = (p.C == 1 ? 0.20 : 0.38) + (p.kn == 1 ? 0.31e-3 : 0.73e-3) * nodes;
+  return 4.0 + waves * (4.0 + nsteps * step);
 }
 
 struct TemporalPlan {
