@@ -630,19 +630,24 @@ static cudaError_t round_launch(const RoundArgs& ra, const Geo& geo, unsigned gr
                       packed, stw);
 }
 
-// Threads per node and tiles per CTA by the number of tiles.  While every tile
-// can have an SM (or half of one) to itself the kernel takes as long as one
-// tile, and four (two) threads per node shorten that; with more tiles than
-// that, one thread per node and four tiles per SM have the higher rate (1024^2
-// step: 0.55 ms, two threads per node 0.58).
+// Threads per node and tiles per CTA by the tiles that an SM gets (whole step
+// of 128 x n lattices, 152 SMs).  One tile: the kernel takes as long as that
+// tile, which four threads per node shorten.  Otherwise one thread per node and
+// four tiles at a time have the higher rate, but an SM then takes its tiles in
+// pairs (a CTA of two groups), so that an odd number costs as much as the next
+// even one; two threads per node and two tiles at a time take them singly:
+// 50 us against 60 for 3 tiles, 72 against 80 for 5, 92 against 101 for 7, 116
+// against 124 for 9, 133 against 140 for 11, 155 against 158 for 13, but 84.5
+// against 80.4 for 6, 127 against 125 for 10, 191 against 184 for 16.
 template <int MODE, bool AH, class Geo>
 static cudaError_t round_t(const RoundArgs& ra, const Geo& geo, int64_t N, int per_sm,
                            const uint8_t* packed, unsigned* stw, cudaStream_t st) {
-  const int64_t ntiles = (N + TILE - 1) / TILE;
-  if (ntiles <= num_sms())
-    return round_launch<MODE, 4, 1, AH>(ra, geo, (unsigned)ntiles, packed, stw, st);
-  if (ntiles <= 2 * num_sms())
-    return round_launch<MODE, 2, 1, AH>(ra, geo, (unsigned)ntiles, packed, stw, st);
+  const int64_t ntiles = (N + TILE - 1) / TILE, sms = num_sms();
+  const int64_t each = (ntiles + sms - 1) / sms;
+  if (each <= 1) return round_launch<MODE, 4, 1, AH>(ra, geo, (unsigned)ntiles, packed, stw, st);
+  if (each == 2 || (each <= 13 && each % 2 == 1))
+    return round_launch<MODE, 2, 1, AH>(ra, geo, (unsigned)(ntiles < 2 * sms ? ntiles : 2 * sms),
+                                        packed, stw, st);
   // persistent grid: at most per_sm CTAs per SM, each running LBM_ROUND_GROUPS tiles at a time
   const int64_t cta_tiles = (ntiles + LBM_ROUND_GROUPS - 1) / LBM_ROUND_GROUPS;
   const unsigned grid = grid_for(cta_tiles * TILE, per_sm >= 2 ? LBM_ROUND_CTAS : per_sm);
