@@ -164,9 +164,16 @@ def register(name, restype, argtypes):
         fn.argtypes = argtypes
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    # (an import statement per argument check cost a few microseconds a call)
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _elems(s):
@@ -232,8 +239,10 @@ def _f64():
 def stream_ptr(stream=None):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream's handle, without the Stream object that
+    # torch.cuda.current_stream() builds around it
+    torch = _torch()
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def check(rc, what=""):
