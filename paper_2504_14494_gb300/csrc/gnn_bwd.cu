@@ -554,13 +554,6 @@ namespace rb2 {
 constexpr uint32_t DAB = 0, H = 32768, ONE = 49152, WABT = 53248, CK = 69632, CKH = 71680,
                    DCR = 72704, SH = 74752, BYTES = 74880;
 }
-#ifndef LBM_RB2_GROUP_A
-#define LBM_RB2_GROUP_A 4  // neighbours whose loads are in flight together, dA side
-#endif
-#ifndef LBM_RB2_GROUP_B
-#define LBM_RB2_GROUP_B 2  // the same, dB side
-#endif
-
 // WALLS (the channel's graph): an edge whose far node lies beyond a wall
 // (row outside [0, ny)) was left out of the forward's sum and passes no
 // gradient; its neighbour address wraps to a row inside, so loads stay in
@@ -569,6 +562,8 @@ constexpr uint32_t DAB = 0, H = 32768, ONE = 49152, WABT = 53248, CK = 69632, CK
 // Bound by the latency of the gathers and of the FP16 chains (FP16 pipe 47 %,
 // issue 45 % with two threads per node at 233 registers: 8 warps); 64 x 256^2
 // training step 11.18 -> 10.85 ms, a step of few tiles 37 -> 31 us per launch.
+// dA and dB direction by direction in one loop (two independent chains)
+// instead of one after the other: 10.85 -> 10.38 ms.
 template <bool WALLS>
 __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
     const __half* __restrict__ ab, const float* __restrict__ da,
@@ -597,6 +592,7 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
   uint8_t* DAB = sm + rb2::DAB;
   uint8_t* H = sm + rb2::H;
   constexpr int NF = 16;  // features of a thread
+  constexpr int GROUP = WALLS ? 1 : 2;  // directions whose loads are in flight together (more spill)
   float dcacc = 0.0f;  // lane l: running sum of value l of [dc_x | dc_y] over this warp's nodes
   const int node = threadIdx.x & 127, part = threadIdx.x >> 7, f0 = part * NF;
   const uint32_t lb = lane_base(tc.tmem);
@@ -609,123 +605,100 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
     const NodeXY p = node_xy(nn, s);
+    const int c0 = f0, ch = c0 >> 3;
+    // 2 GELU'(z) is evaluated in packed FP16 pairs (z = A + B + c_k is O(1)).
+    // dA_j = da_j * sum_k GELU'(z_jk) factors: the sums over k (and their
+    // e_kx / e_ky weighted forms) are taken in FP16 and multiplied by da_j
+    // once.  dB_j needs the neighbours' da, so its terms are accumulated in
+    // FP32 (gradients would underflow FP16).  Direction k of both sides goes
+    // through together: two independent chains per pair of features.
+    uint32_t aj[8], bj[8];
     {
-      const int c0 = f0, ch = c0 >> 3;
-      // 2 GELU'(z) is evaluated in packed FP16 pairs (z = A + B + c_k is O(1)).
-      // dA_j = da_j * sum_k GELU'(z_jk) factors: the sums over k (and their
-      // e_kx / e_ky weighted forms) are taken in FP16 and multiplied by da_j
-      // once.  dB_j needs the neighbours' da, so its terms are accumulated in
-      // FP32 (gradients would underflow FP16).  The two halves run one after
-      // the other to keep few values live.
-      {  // dA_j and dc_j over the neighbours j + e_k
-        uint32_t aj[8];
-        {
-          const uint4 a0 = __ldg(chunk8(ab, N, nn, c0)), a1 = __ldg(chunk8(ab, N, nn, c0 + 8));
-          aj[0] = a0.x; aj[1] = a0.y; aj[2] = a0.z; aj[3] = a0.w;
-          aj[4] = a1.x; aj[5] = a1.y; aj[6] = a1.z; aj[7] = a1.w;
-        }
-        __half2 S[8], Sx[8], Sy[8];  // sums over k of 2 GELU'(z_jk), e_kx and e_ky weighted
+      const uint4 a0 = __ldg(chunk8(ab, N, nn, c0)), a1 = __ldg(chunk8(ab, N, nn, c0 + 8));
+      aj[0] = a0.x; aj[1] = a0.y; aj[2] = a0.z; aj[3] = a0.w;
+      aj[4] = a1.x; aj[5] = a1.y; aj[6] = a1.z; aj[7] = a1.w;
+      const uint4 b0 = __ldg(chunk8(ab, N, nn, HID + c0));
+      const uint4 b1 = __ldg(chunk8(ab, N, nn, HID + c0 + 8));
+      bj[0] = b0.x; bj[1] = b0.y; bj[2] = b0.z; bj[3] = b0.w;
+      bj[4] = b1.x; bj[5] = b1.y; bj[6] = b1.z; bj[7] = b1.w;
+    }
+    __half2 S[8], Sx[8], Sy[8];  // sums over k of 2 GELU'(z_jk), e_kx and e_ky weighted
+    float gB[16];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) S[c] = Sx[c] = Sy[c] = __float2half2_rn(0.0f);
+    for (int c = 0; c < 8; ++c) S[c] = Sx[c] = Sy[c] = __float2half2_rn(0.0f);
 #pragma unroll
-        for (int g = 0; g < 8; g += LBM_RB2_GROUP_A) {  // directions k = g+1 .. g+LBM_RB2_GROUP_A
-          uint4 bn[LBM_RB2_GROUP_A][2];
+    for (int c = 0; c < 16; ++c) gB[c] = 0.0f;
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP_A; ++kk) {
-            const int k = g + kk + 1;
-            const int64_t j = checked(node_at(p, ex(k), ey(k), s), 0, N, stw);
-            bn[kk][0] = __ldg(chunk8(ab, N, j, HID + c0));
-            bn[kk][1] = __ldg(chunk8(ab, N, j, HID + c0 + 8));
-          }
+    for (int g = 0; g < 8; g += GROUP) {  // directions k = g+1 .. g+GROUP
+      uint4 bn[GROUP][2], ai[GROUP][2];
+      float4 di[GROUP][4];
 #pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP_A; ++kk) {
-            const int k = g + kk + 1;
-            const __half2* c_k = ckh + (k - 1) * (HID / 2) + c0 / 2;
-            const uint32_t* bw = reinterpret_cast<const uint32_t*>(bn[kk]);
-            const bool keep = !WALLS || (unsigned)(p.y + ey(k)) < (unsigned)s.ny;
+      for (int kk = 0; kk < GROUP; ++kk) {
+        const int k = g + kk + 1;
+        const int64_t j = checked(node_at(p, ex(k), ey(k), s), 0, N, stw);    // dA: B of j + e_k
+        bn[kk][0] = __ldg(chunk8(ab, N, j, HID + c0));
+        bn[kk][1] = __ldg(chunk8(ab, N, j, HID + c0 + 8));
+        const int64_t i = checked(node_at(p, -ex(k), -ey(k), s), 0, N, stw);  // dB: A, da of j - e_k
+        ai[kk][0] = __ldg(chunk8(ab, N, i, c0));
+        ai[kk][1] = __ldg(chunk8(ab, N, i, c0 + 8));
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const __half2 z = __hadd2(__hadd2(u32_as_h2(aj[c]), c_k[c]), u32_as_h2(bw[c]));
-              const __half2 gp = keep ? gelu_grad2_h2(z) : __float2half2_rn(0.0f);
-              S[c] = __hadd2(S[c], gp);
-              if (ex(k) > 0) Sx[c] = __hadd2(Sx[c], gp);
-              if (ex(k) < 0) Sx[c] = __hsub2(Sx[c], gp);
-              if (ey(k) > 0) Sy[c] = __hadd2(Sy[c], gp);
-              if (ey(k) < 0) Sy[c] = __hsub2(Sy[c], gp);
-            }
-          }
-        }
-        float gA[16], v[32];  // v = [dc_x | dc_y] of this node
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 t = __ldg(chunk4(da, N, nn, c0 + 4 * i));
-          const float dd[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {  // the factor 1/2 of 2 GELU' is applied here
-            const int c = 4 * i + q;
-            const float d = on ? 0.5f * dd[q] : 0.0f;
-            const float2 sv = __half22float2(S[c >> 1]), sx = __half22float2(Sx[c >> 1]);
-            const float2 sy = __half22float2(Sy[c >> 1]);
-            gA[c] = d * ((c & 1) ? sv.y : sv.x);
-            v[c] = d * ((c & 1) ? sx.y : sx.x);
-            v[16 + c] = d * ((c & 1) ? sy.y : sy.x);
-          }
-        }
-        *reinterpret_cast<uint4*>(DAB + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gA);
-        *reinterpret_cast<uint4*>(DAB + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
-            pack_bf16x8(gA + 8);
-        // dc sums over this warp's 32 nodes: lane l gets value l of [dc_x | dc_y]
-        dcacc += warp_transpose_sum(v);
+        for (int t4 = 0; t4 < 4; ++t4) di[kk][t4] = __ldg(chunk4(da, N, i, c0 + 4 * t4));
       }
-      {  // dB_j over the neighbours i = j - e_k
-        uint32_t bj[8];
-        {
-          const uint4 b0 = __ldg(chunk8(ab, N, nn, HID + c0));
-          const uint4 b1 = __ldg(chunk8(ab, N, nn, HID + c0 + 8));
-          bj[0] = b0.x; bj[1] = b0.y; bj[2] = b0.z; bj[3] = b0.w;
-          bj[4] = b1.x; bj[5] = b1.y; bj[6] = b1.z; bj[7] = b1.w;
+#pragma unroll
+      for (int kk = 0; kk < GROUP; ++kk) {
+        const int k = g + kk + 1;
+        const __half2* c_k = ckh + (k - 1) * (HID / 2) + c0 / 2;
+        const uint32_t* bw = reinterpret_cast<const uint32_t*>(bn[kk]);
+        const uint32_t* aw = reinterpret_cast<const uint32_t*>(ai[kk]);
+        const float* dv = reinterpret_cast<const float*>(di[kk]);
+        // walls: the edges (j, k) and (j - e_k, k) exist if their far nodes lie inside
+        const bool keep_a = !WALLS || (unsigned)(p.y + ey(k)) < (unsigned)s.ny;
+        const bool keep_b = !WALLS || (unsigned)(p.y - ey(k)) < (unsigned)s.ny;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const __half2 z = __hadd2(__hadd2(u32_as_h2(aj[c]), c_k[c]), u32_as_h2(bw[c]));
+          const __half2 gp = keep_a ? gelu_grad2_h2(z) : __float2half2_rn(0.0f);
+          S[c] = __hadd2(S[c], gp);
+          if (ex(k) > 0) Sx[c] = __hadd2(Sx[c], gp);
+          if (ex(k) < 0) Sx[c] = __hsub2(Sx[c], gp);
+          if (ey(k) > 0) Sy[c] = __hadd2(Sy[c], gp);
+          if (ey(k) < 0) Sy[c] = __hsub2(Sy[c], gp);
+          const __half2 w = __hadd2(__hadd2(u32_as_h2(aw[c]), c_k[c]), u32_as_h2(bj[c]));
+          const float2 gq = keep_b ? __half22float2(gelu_grad2_h2(w)) : make_float2(0.0f, 0.0f);
+          gB[2 * c] = fmaf(dv[2 * c], gq.x, gB[2 * c]);
+          gB[2 * c + 1] = fmaf(dv[2 * c + 1], gq.y, gB[2 * c + 1]);
         }
-        float gB[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) gB[c] = 0.0f;
-#pragma unroll
-        for (int g = 0; g < 8; g += LBM_RB2_GROUP_B) {
-          uint4 ai[LBM_RB2_GROUP_B][2];
-          float4 di[LBM_RB2_GROUP_B][4];
-#pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP_B; ++kk) {
-            const int k = g + kk + 1;
-            const int64_t i = checked(node_at(p, -ex(k), -ey(k), s), 0, N, stw);
-            ai[kk][0] = __ldg(chunk8(ab, N, i, c0));
-            ai[kk][1] = __ldg(chunk8(ab, N, i, c0 + 8));
-#pragma unroll
-            for (int t4 = 0; t4 < 4; ++t4) di[kk][t4] = __ldg(chunk4(da, N, i, c0 + 4 * t4));
-          }
-#pragma unroll
-          for (int kk = 0; kk < LBM_RB2_GROUP_B; ++kk) {
-            const int k = g + kk + 1;
-            const __half2* c_k = ckh + (k - 1) * (HID / 2) + c0 / 2;
-            const uint32_t* aw = reinterpret_cast<const uint32_t*>(ai[kk]);
-            const float* dv = reinterpret_cast<const float*>(di[kk]);
-            // the edge (i, k) into this node exists if i lies inside
-            const bool keep = !WALLS || (unsigned)(p.y - ey(k)) < (unsigned)s.ny;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const __half2 z = __hadd2(__hadd2(u32_as_h2(aw[c]), c_k[c]), u32_as_h2(bj[c]));
-              const float2 gp = keep ? __half22float2(gelu_grad2_h2(z)) : make_float2(0.0f, 0.0f);
-              gB[2 * c] = fmaf(dv[2 * c], gp.x, gB[2 * c]);
-              gB[2 * c + 1] = fmaf(dv[2 * c + 1], gp.y, gB[2 * c + 1]);
-            }
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < 16; ++c) gB[c] = on ? 0.5f * gB[c] : 0.0f;
-        uint8_t* b1 = DAB + 16384;
-        *reinterpret_cast<uint4*>(b1 + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gB);
-        *reinterpret_cast<uint4*>(b1 + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
-            pack_bf16x8(gB + 8);
       }
     }
+    {
+      float gA[16], v[32];  // v = [dc_x | dc_y] of this node
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 t = __ldg(chunk4(da, N, nn, c0 + 4 * i));
+        const float dd[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {  // the factor 1/2 of 2 GELU' is applied here
+          const int c = 4 * i + q;
+          const float d = on ? 0.5f * dd[q] : 0.0f;
+          const float2 sv = __half22float2(S[c >> 1]), sx = __half22float2(Sx[c >> 1]);
+          const float2 sy = __half22float2(Sy[c >> 1]);
+          gA[c] = d * ((c & 1) ? sv.y : sv.x);
+          v[c] = d * ((c & 1) ? sx.y : sx.x);
+          v[16 + c] = d * ((c & 1) ? sy.y : sy.x);
+        }
+      }
+      *reinterpret_cast<uint4*>(DAB + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gA);
+      *reinterpret_cast<uint4*>(DAB + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
+          pack_bf16x8(gA + 8);
+      // dc sums over this warp's 32 nodes: lane l gets value l of [dc_x | dc_y]
+      dcacc += warp_transpose_sum(v);
+    }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) gB[c] = on ? 0.5f * gB[c] : 0.0f;
+    uint8_t* b1 = DAB + 16384;
+    *reinterpret_cast<uint4*>(b1 + node * 128 + ((ch ^ (node & 7)) << 4)) = pack_bf16x8(gB);
+    *reinterpret_cast<uint4*>(b1 + node * 128 + (((ch + 1) ^ (node & 7)) << 4)) =
+        pack_bf16x8(gB + 8);
     copy_row<NF>(H, node, f0, h_in, N, nn);
     const bool acc = !first;
     if (!tc_run(sh, tc, stw, [&] {
