@@ -32,9 +32,9 @@ template <int NT, int NPT>
 __global__ void __launch_bounds__(NT) bgk_batch_kernel(const float* __restrict__ fin,
                                                        float* __restrict__ fout,
                                                        const LatDesc* __restrict__ lat, int nlat,
-                                                       const int* __restrict__ hint, int64_t count,
+                                                       const LatBlock* __restrict__ block, int64_t count,
                                                        int64_t ps, unsigned* stw) {
-  const GeoTable geo{lat, 0, nlat, 0, count, ps, hint};
+  const GeoTable geo{lat, 0, nlat, 0, count, ps, block};
   const int64_t g0 = (int64_t)blockIdx.x * (NT * NPT) + threadIdx.x;
   float f[NPT][Q];
   int b[NPT];
@@ -151,28 +151,28 @@ const std::vector<int> kBgkTiles = {1281, 1282, 1284, 2561, 2562, 2564, 5121, 51
 
 template <int NT, int NPT>
 static void bgk_batch_t(const float* fin, float* fout, const LatDesc* lat, int nlat,
-                        const int* hint, int64_t count, int64_t ps, unsigned* stw,
+                        const LatBlock* block, int64_t count, int64_t ps, unsigned* stw,
                         cudaStream_t st) {
   const int64_t per = (int64_t)NT * NPT;
   bgk_batch_kernel<NT, NPT><<<(unsigned)((count + per - 1) / per), NT, 0, st>>>(
-      fin, fout, lat, nlat, hint, count, ps, stw);
+      fin, fout, lat, nlat, block, count, ps, stw);
 }
 
 cudaError_t launch_bgk_batch(const float* fin, float* fout, const LatDesc* lat, int nlat,
-                             const int* hint, int64_t count, int64_t ps, int tile,
+                             const LatBlock* block, int64_t count, int64_t ps, int tile,
                              cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   switch (tile) {
-    case 1281: bgk_batch_t<128, 1>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 1282: bgk_batch_t<128, 2>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 1284: bgk_batch_t<128, 4>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 2562: bgk_batch_t<256, 2>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 2564: bgk_batch_t<256, 4>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 5121: bgk_batch_t<512, 1>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    case 5122: bgk_batch_t<512, 2>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
-    default: bgk_batch_t<256, 1>(fin, fout, lat, nlat, hint, count, ps, stw, st); break;
+    case 1281: bgk_batch_t<128, 1>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 1282: bgk_batch_t<128, 2>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 1284: bgk_batch_t<128, 4>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 2562: bgk_batch_t<256, 2>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 2564: bgk_batch_t<256, 4>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 5121: bgk_batch_t<512, 1>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    case 5122: bgk_batch_t<512, 2>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
+    default: bgk_batch_t<256, 1>(fin, fout, lat, nlat, block, count, ps, stw, st); break;
   }
   return cudaGetLastError();
 }
@@ -185,7 +185,7 @@ struct lbm_batch_plan {
   int n = 0, n_bgk = 0, n_gnn = 0;
   std::vector<int64_t> offset_of_input;  // first node of input lattice i
   LatDesc* d_lat = nullptr;               // sorted: BGK group, then GNN group
-  int* d_hint = nullptr;                  // per 128-node block: lattice of its first node
+  LatBlock* d_block = nullptr;            // per 128-node block: the lattice of its first node
   double* d_prm = nullptr;                // [n][4] TGV parameters (sorted order)
   std::vector<int> sorted_to_input;
   int64_t bgk_nodes = 0, gnn_nodes = 0, total = 0;
@@ -208,7 +208,7 @@ void plan_release(lbm_batch_plan* p) {
   if (p->cap) cudaStreamDestroy(p->cap);
   if (p->side) cudaStreamDestroy(p->side);
   if (p->d_lat) cudaFree(p->d_lat);
-  if (p->d_hint) cudaFree(p->d_hint);
+  if (p->d_block) cudaFree(p->d_block);
   if (p->d_prm) cudaFree(p->d_prm);
   delete p;
 }
@@ -220,13 +220,13 @@ cudaError_t plan_step(lbm_batch_plan* p, const float* src, float* dst, const uin
                       __nv_bfloat16* ws, cudaStream_t s_bgk, cudaStream_t s_gnn) {
   cudaError_t e = cudaSuccess;
   if (p->n_bgk > 0) {
-    e = launch_bgk_batch(src, dst, p->d_lat, p->n_bgk, p->d_hint, p->bgk_nodes, p->total,
+    e = launch_bgk_batch(src, dst, p->d_lat, p->n_bgk, p->d_block, p->bgk_nodes, p->total,
                          p->bgk_block,
                          s_bgk);
     if (e != cudaSuccess) return e;
   }
   if (p->n_gnn > 0) {
-    e = launch_gnn_step_table(src, dst, p->d_lat, p->n_bgk, p->n_gnn, p->d_hint, p->bgk_nodes,
+    e = launch_gnn_step_table(src, dst, p->d_lat, p->n_bgk, p->n_gnn, p->d_block, p->bgk_nodes,
                               p->gnn_nodes,
                               p->total, packed, ws, s_gnn, p->gnn_per_sm);
   }
@@ -277,16 +277,17 @@ int lbm_batch_plan_create(const lbm_lattice_desc* lattices, int n, lbm_batch_pla
     return LBM_ERR_SIZE;
   }
   // lattice of the first node of every 128-node block
-  std::vector<int> hint((size_t)((p->total + 127) / 128));
-  for (size_t blk = 0, lo = 0; blk < hint.size(); ++blk) {
+  std::vector<LatBlock> block((size_t)((p->total + 127) / 128));
+  for (size_t blk = 0, lo = 0; blk < block.size(); ++blk) {
     const int64_t g = (int64_t)blk * 128;
     while (lo + 1 < table.size() && table[lo + 1].offset <= g) ++lo;
-    hint[blk] = (int)lo;
+    const int64_t next = lo + 1 < table.size() ? table[lo + 1].offset : p->total;
+    block[blk] = {table[lo].offset, next, table[lo].nx, table[lo].ny, (int32_t)lo, 0};
   }
   if (cudaGetDevice(&p->device) != cudaSuccess ||
       cudaMalloc(&p->d_lat, sizeof(LatDesc) * n) != cudaSuccess ||
-      cudaMalloc(&p->d_hint, sizeof(int) * hint.size()) != cudaSuccess ||
-      cudaMemcpy(p->d_hint, hint.data(), sizeof(int) * hint.size(), cudaMemcpyHostToDevice) !=
+      cudaMalloc(&p->d_block, sizeof(LatBlock) * block.size()) != cudaSuccess ||
+      cudaMemcpy(p->d_block, block.data(), sizeof(LatBlock) * block.size(), cudaMemcpyHostToDevice) !=
           cudaSuccess ||
       cudaMalloc(&p->d_prm, sizeof(double) * 4 * n) != cudaSuccess ||
       cudaMemcpy(p->d_lat, table.data(), sizeof(LatDesc) * n, cudaMemcpyHostToDevice) !=
@@ -360,7 +361,7 @@ int lbm_batch_run(lbm_batch_plan* plan, const float* f_in, float* f_out, float* 
   if (!plan->bgk_block) {
     plan->bgk_block = plan->n_bgk == 0 ? 2561 : tune("bgk_batch_tile", plan->bgk_nodes, kBgkTiles, st,
         [&](int c) {
-          return launch_bgk_batch(f_in, f_out, plan->d_lat, plan->n_bgk, plan->d_hint,
+          return launch_bgk_batch(f_in, f_out, plan->d_lat, plan->n_bgk, plan->d_block,
                                   plan->bgk_nodes,
                                   plan->total, c, st);
         });
@@ -369,7 +370,7 @@ int lbm_batch_run(lbm_batch_plan* plan, const float* f_in, float* f_out, float* 
     plan->gnn_per_sm = plan->n_gnn == 0 ? 2 : tune("gnn_step_table", plan->gnn_nodes, {1, 2}, st,
         [&](int c) {
           return launch_gnn_step_table(f_in, f_out, plan->d_lat, plan->n_bgk, plan->n_gnn,
-                                       plan->d_hint, plan->bgk_nodes, plan->gnn_nodes, plan->total, pk, ws, st,
+                                       plan->d_block, plan->bgk_nodes, plan->gnn_nodes, plan->total, pk, ws, st,
                                        c);
         });
   }

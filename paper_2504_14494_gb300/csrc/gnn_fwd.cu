@@ -716,18 +716,18 @@ cudaError_t launch_gnn_forward_channel(const float* f_pre, const Shape& s, float
 }
 
 cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc* lat, int first,
-                                  int n, const int* hint, int64_t base, int64_t count, int64_t ps,
+                                  int n, const LatBlock* block, int64_t base, int64_t count, int64_t ps,
                                   const uint8_t* packed, __nv_bfloat16* ws, cudaStream_t st,
                                   int per_sm) {
   if (count <= 0) return cudaSuccess;
-  const GeoTable geo{lat, first, n, base, count, ps, hint};
+  const GeoTable geo{lat, first, n, base, count, ps, block};
   __nv_bfloat16* h0 = ws;
   __half* b0 = reinterpret_cast<__half*>(h0 + count * 64);
   __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(b0 + count * 64);
   __half* b1 = reinterpret_cast<__half*>(h1 + count * 64);
   cudaError_t e;
   // the whole step of an MLP-only network, or the encoder (gnn_mlp.cu)
-  if ((e = launch_gnn_encode_fused_table(f_in, f_out, lat, first, n, hint, base, count, ps, packed,
+  if ((e = launch_gnn_encode_fused_table(f_in, f_out, lat, first, n, block, base, count, ps, packed,
                                          h0, b0, st)) != cudaSuccess)
     return e;
   RoundLaunch r0;

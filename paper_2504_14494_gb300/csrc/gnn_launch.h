@@ -74,6 +74,7 @@ cudaError_t launch_gnn_mlp_step(const float* f_in, float* f_out, const Shape& s,
                                 const float* taus, const uint8_t* packed, cudaStream_t st);
 
 struct LatDesc;
+struct LatBlock;
 // The first launch of a GNN-LBM step, for whichever network the image holds:
 // for the MLP-only network its whole step (the round kernels then return at
 // once), else the inference encoder in the same design (pull, features, two
@@ -84,17 +85,16 @@ cudaError_t launch_gnn_encode_fused(const float* f_in, float* f_out, const Shape
                                     const float* taus, const uint8_t* packed, __nv_bfloat16* h0,
                                     __half* b, cudaStream_t st);
 cudaError_t launch_gnn_encode_fused_table(const float* f_in, float* f_out, const LatDesc* lat,
-                                          int first, int n, const int* hint, int64_t base,
+                                          int first, int n, const LatBlock* block, int64_t base,
                                           int64_t count, int64_t ps, const uint8_t* packed,
                                           __nv_bfloat16* h0, __half* b, cudaStream_t st);
 // GNN-LBM step (encoder, 2 rounds, head + Eq. 3) on the lattices first ..
 // first+n-1 of a device descriptor table, whose nodes are [base, base+count)
-// of population buffers with plane stride ps; hint: device int per 128-node
-// block of the buffers, the lattice holding the block's first node (or
-// NULL: binary search); ws: count * 512 bytes; per_sm: resident CTAs per SM
-// of the persistent grids.
+// of population buffers with plane stride ps; block: device entry per
+// 128-node block of the buffers (or NULL: binary search); ws: count * 512
+// bytes; per_sm: resident CTAs per SM of the persistent grids.
 cudaError_t launch_gnn_step_table(const float* f_in, float* f_out, const LatDesc* lat, int first,
-                                  int n, const int* hint, int64_t base, int64_t count, int64_t ps,
+                                  int n, const LatBlock* block, int64_t base, int64_t count, int64_t ps,
                                   const uint8_t* packed, __nv_bfloat16* ws, cudaStream_t st,
                                   int per_sm);
 

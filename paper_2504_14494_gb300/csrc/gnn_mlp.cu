@@ -593,10 +593,10 @@ cudaError_t launch_gnn_encode_fused(const float* f_in, float* f_out, const Shape
 }
 
 cudaError_t launch_gnn_encode_fused_table(const float* f_in, float* f_out, const LatDesc* lat,
-                                          int first, int n, const int* hint, int64_t base,
+                                          int first, int n, const LatBlock* block, int64_t base,
                                           int64_t count, int64_t ps, const uint8_t* packed,
                                           __nv_bfloat16* h0, __half* b, cudaStream_t st) {
-  return step_first(MlpArgs<GeoTable>{f_in, f_out, GeoTable{lat, first, n, base, count, ps, hint},
+  return step_first(MlpArgs<GeoTable>{f_in, f_out, GeoTable{lat, first, n, base, count, ps, block},
                                       0.0f, nullptr, packed, false, h0, b, nullptr},
                     count, st);
 }
