@@ -26,7 +26,8 @@
 // times recomputed nodes; 1024^2: 8.4 (10.6); 512^2: 4.2 (6.2); 256^2: 2.6
 // (4.2); three odd 1023 x 517: 12.3 (22.8).  Tried on the way: one thread per
 // node with all stages handed over in shared memory, 119 at 4096^2; 4 columns
-// per lane, 79 to 83 (fewer warps, and the barrier or the registers bind).
+// per lane, 79 to 83 (fewer warps, and the barrier or the registers bind); a
+// warp's stages in two independent groups, one a row late, 74 (204 registers).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
