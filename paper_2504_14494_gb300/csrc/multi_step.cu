@@ -7,11 +7,11 @@
 // Two forms, chosen by estimated time (launch_bgk_steps):
 //
 // resident_steps_kernel -- for small lattices and many steps, which are bound
-// by the latency of one step: one thread-block cluster (1..8 CTAs) per lattice
+// by the latency of one step: one thread-block cluster (1..16 CTAs) per lattice
 // holds the whole lattice in shared memory (two buffers) for all steps of the
 // call; per step a pull from shared memory, the collision, a store to the
 // other buffer, edge rows also to the neighbouring CTAs' halo rows through
-// distributed shared memory.  64^2: 0.54 us a step (4.1 with one launch a
+// distributed shared memory.  64^2: 0.41 us a step (4.1 with one launch a
 // step); a 4 x 32 channel, in one CTA: 0.23 (4.1).
 //
 // temporal_steps_kernel -- for larger lattices, which are bound by memory
@@ -225,16 +225,13 @@ constexpr int SMEM_MAX = 227 * 1024 - 64;  // (64: the mbarriers)
 
 uint32_t resident_smem(int rows, int nx) { return 2u * Q * (uint32_t)(rows + 2) * nx * 4u; }
 
-// Cluster size and rows per CTA, or C = 0 when the lattice does not fit.  Up to
-// 512 nodes one CTA without an exchange is faster than several (8 x 32 channel:
-// 0.26 us a step against 0.44), above that the largest cluster.
+// Cluster size (the largest up to C that leaves no CTA without rows) and rows
+// per CTA, or C = 0 when the lattice does not fit.
 struct ResidentPlan {
   int C, rows, threads, kn;
 };
-ResidentPlan plan_resident(const Shape& s) {
-  const int64_t all = (int64_t)s.nx * s.ny;
-  if (all > 8 * 3072) return {0, 0, 0, 0};
-  for (int C = all <= 512 ? 1 : 8; C >= 1; C >>= 1) {
+ResidentPlan plan_resident_from(const Shape& s, int C) {
+  for (; C >= 1; C >>= 1) {
     if (C > s.ny) continue;
     const int rows = (s.ny + C - 1) / C;
     if ((int64_t)rows * (C - 1) >= s.ny) continue;  // a CTA without rows
@@ -255,6 +252,9 @@ cudaError_t resident_t(const ResidentArgs& a, const ResidentPlan& p, cudaStream_
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
+  if (p.C > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                           1)) != cudaSuccess)
+    return e;
   cfg.gridDim = dim3((unsigned)p.C * (unsigned)a.s.nb);
   cfg.blockDim = dim3((unsigned)p.threads);
   cfg.dynamicSmemBytes = bytes;
@@ -497,16 +497,69 @@ double single_us(const Shape& s) {
   return std::max({4.1, 3.0 + 7.3e-6 * n, 10.45e-6 * n});
 }
 
+// Clusters of 16 CTAs (more than every device takes) that run at once on this
+// one, at the kernel's most threads and shared memory; 0: none.
+int clusters16() {
+  static std::atomic<int> cached[64];  // + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    auto* kern = resident_steps_kernel<false, 1, false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = SMEM_MAX;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 16;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int most = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&most, kern, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      most = 0;
+    }
+    n = most + 1;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n - 1;
+}
+
 // `nsteps` steps of the resident form: 4 for the launch; per wave of clusters
-// (about 16 of 8 CTAs run at once) 4 to load and store; per step the chain of
-// one node and the exchange, and the nodes of a CTA (more than one per thread
-// at half the rate).
+// (about 16 of 8 CTAs run at once, of 16 CTAs what the device says) 4 to load
+// and store; per step the chain of one node and the exchange, and the nodes of
+// a CTA (more than one per thread at half the rate; clusters of 16 fitted by
+// themselves: 64^2, 100 x 96, 128^2, 200^2).
 double resident_us(const Shape& s, const ResidentPlan& p, int nsteps) {
-  const int at_once = 128 / p.C;
+  const int at_once = p.C == 16 ? std::max(1, clusters16()) : 128 / p.C;
   const double waves = (double)((s.nb + at_once - 1) / at_once);
   const double nodes = (double)p.rows * s.nx;
-  const double step = (p.C == 1 ? 0.20 : 0.38) + (p.kn == 1 ? 0.31e-3 : 0.73e-3) * nodes;
+  const double step = p.C == 16 ? std::max(0.37, 0.24 + (p.kn == 1 ? 0.64e-3 : 0.91e-3) * nodes)
+                                : (p.C == 1 ? 0.20 : 0.38) + (p.kn == 1 ? 0.31e-3 : 0.73e-3) * nodes;
   return 4.0 + waves * (4.0 + nsteps * step);
+}
+
+// The fastest by that estimate.  One CTA up to 512 nodes without an exchange
+// beats several (8 x 32 channel: 0.26 us a step against 0.44).  Clusters of 16
+// halve the nodes of a CTA: 64^2 0.41 us a step against 0.53 in clusters of 8,
+// 128^2 1.09 against 2.08 (several steps per pass), four 100 x 96 1.05 against
+// 1.69; at 32^2 nothing is left to halve (0.38 against 0.36), and fewer run at
+// once (one per GPC), so that stacks stay with 8.
+ResidentPlan plan_resident(const Shape& s, int nsteps) {
+  const int64_t all = (int64_t)s.nx * s.ny;
+  if (all > 16 * 3072) return {0, 0, 0, 0};
+  ResidentPlan p = plan_resident_from(s, all <= 512 ? 1 : 8);
+  if (all > 1024 && s.ny >= 16 && clusters16() > 0) {
+    const ResidentPlan w = plan_resident_from(s, 16);
+    if (w.C == 16 && (!p.C || resident_us(s, w, nsteps) < resident_us(s, p, nsteps))) p = w;
+  }
+  return p;
 }
 
 struct TemporalPlan {
@@ -611,7 +664,7 @@ cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const S
   passes = head;
   for (int n = left; n > 0; n -= first[n]) ++passes;
 
-  const ResidentPlan rp = plan_resident(s);
+  const ResidentPlan rp = plan_resident(s, nsteps);
   if (rp.C && resident_us(s, rp, nsteps) < total) {
     const ResidentArgs a{fin, fout, s, tau, taus, 0.0f, nsteps, rp.rows};
     return resident<false>(a, rp, st);
@@ -638,14 +691,14 @@ cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const S
 // The channel has the resident form alone; its single-step kernel takes 4.2 a
 // launch, 16.7e-6 per node.
 bool channel_steps_fit(const Shape& s, int nsteps) {
-  const ResidentPlan rp = plan_resident(s);
+  const ResidentPlan rp = plan_resident(s, nsteps);
   const double single = std::max(4.2, 16.7e-6 * (double)s.nb * s.ny * s.nx);
   return rp.C != 0 && 1.1 * resident_us(s, rp, nsteps) < 4.0 + nsteps * single;
 }
 
 cudaError_t launch_channel_steps(const float* fin, float* fout, const Shape& s, float tau,
                                  const float* taus, float gx, int nsteps, cudaStream_t st) {
-  const ResidentPlan rp = plan_resident(s);
+  const ResidentPlan rp = plan_resident(s, nsteps);
   if (!rp.C) return cudaErrorInvalidValue;
   const ResidentArgs a{fin, fout, s, tau, taus, gx, nsteps, rp.rows};
   return resident<true>(a, rp, st);

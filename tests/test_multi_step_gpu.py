@@ -75,3 +75,23 @@ def test_totals_of_the_last_state(lbmlib, cuda, nx, ny, nb):
         scale = want[0].item()
         assert np.abs((t - want).cpu().numpy()).max() <= 1e-12 * scale
     assert L.lbm_get_status() == 0
+
+
+@pytest.mark.parametrize("nx,ny,nb", [(64, 16, 1), (61, 17, 1), (37, 31, 2), (128, 128, 1), (190, 250, 1),
+                                      (3, 3000, 1), (191, 256, 1), (96, 96, 20)])
+def test_clusters_of_sixteen_equal_single_steps(lbmlib, cuda, nx, ny, nb):
+    import torch
+    L = lbmlib
+    n = nx * ny * nb
+    s = L.shape(nx, ny, nb)
+    for steps in (2, 25):
+        for call, more in ((L.lbm_step_bgk, ()), (L.lbm_step_channel, (1e-4,))):
+            f = _state(n, n, cuda, seed=nx + steps)
+            out, tmp = torch.empty_like(f), torch.empty_like(f)
+            call(f, out, tmp, s, 0.7, None, *more, nsteps=steps)
+            a, b = f.clone(), torch.empty_like(f)
+            for _ in range(steps):
+                call(a, b, None, s, 0.7, None, *more, nsteps=1)
+                a, b = b, a
+            assert _same(out, a, n, n), (call.__name__, steps)
+    assert L.lbm_get_status() == 0
