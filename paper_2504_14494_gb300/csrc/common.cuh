@@ -196,17 +196,31 @@ struct Shape {
 // ---- kernels of one call that overlap at their seams -------------------------
 // The kernels of a multi-kernel call are launched with programmatic stream
 // serialization (launch_after, launch.h): a kernel starts once every CTA of the
-// one before it has passed dep_sync(), reads what no kernel of the call writes
-// but the one before the last or an earlier call (the weights), sets up, and
-// waits in dep_sync() until the one before it has completed and its writes are
-// visible.  Each kernel passes dep_sync() on every path, before it reads or
-// writes anything else, so that "the one before has completed" holds for all
-// before it.  The first kernel of a call is launched normally.
-__device__ __forceinline__ void dep_sync() {
+// one before it has passed dep_release(), sets up from what was complete by
+// then (the weights), and waits in dep_wait() until the one before it has
+// completed and its writes are visible.  Each kernel passes dep_wait() on every
+// path, before dep_release(), before it reads anything the one before may have
+// written and before it writes anything but the status word, so that "the one
+// before has completed" holds for all before it.  gnn_pack, gnn_adamw,
+// gnn_backward and gnn_collide_loss launch their first kernel this way too (it
+// waits before its first read); the first kernel of every other call is
+// launched normally.
+// A kernel allocates its tensor memory before dep_release(): CTAs of the next
+// kernel allocate theirs before they wait, and one that took columns of an SM
+// from a CTA it waits for would block both for good.
+__device__ __forceinline__ void dep_wait() {
 #if __CUDA_ARCH__ >= 900
   asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void dep_release() {
+#if __CUDA_ARCH__ >= 900
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void dep_sync() {
+  dep_wait();
+  dep_release();
 }
 
 }  // namespace lbmgnn

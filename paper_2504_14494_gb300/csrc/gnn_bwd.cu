@@ -343,7 +343,7 @@ constexpr uint32_t XT = 0, ONE = 32768, H2 = 36864, WHF = 53248, DYS = 55808, SH
 __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
     const float* __restrict__ dy, const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh,
     float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
-  dep_sync();  // before the weights: as a call's first kernel it may follow their pack
+  dep_wait();  // before the weights: as a call's first kernel it may follow their pack
   if (!blob_ok(packed, stw)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
   ones_row(sm + hb::ONE, 16, 0);
   TcCtx tc;
   tc_setup(sh, tc);
+  dep_release();
   const float* whf = reinterpret_cast<const float*>(sm + hb::WHF);
   float* dys = reinterpret_cast<float*>(sm + hb::DYS);
   uint8_t* XT = sm + hb::XT;

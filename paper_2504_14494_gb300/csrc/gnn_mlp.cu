@@ -156,7 +156,8 @@ __device__ __forceinline__ void gelu_to_tmem(uint32_t lane_d, uint32_t lane_a,
 // network: the same pull, features and first two layers with GELU, then the
 // round-0 edge term B = W_b h0; h0 (BF16) and B (FP16) go to HBM in the
 // chunked plane layout of the round kernels.
-template <class Geo, bool ENC>
+// RELEASE: the next kernel may start once the tensor memory is allocated.
+template <class Geo, bool ENC, bool RELEASE>
 __device__ __forceinline__ void mlp_or_encode(
     const float* __restrict__ f_in, float* __restrict__ f_out, const Geo& geo, float tau0,
     const float* __restrict__ taus, const uint8_t* __restrict__ packed, int variant, bool rows,
@@ -321,6 +322,7 @@ __device__ __forceinline__ void mlp_or_encode(
   tc_fence_before();
   __syncthreads();  // (also publishes the shared-memory writes above)
   tc_fence_after();
+  if constexpr (RELEASE) dep_release();
   TcCtx tc;
   tc.bar = &sh[grp].bar;  // the group's own mbarrier; its slice of the columns:
   tc.phase = 0;
@@ -514,8 +516,8 @@ struct MlpArgs {
 // cost the encoder 3 us at 1024^2.
 template <class Geo>
 __device__ __noinline__ void mlp_only_step(const MlpArgs<Geo>* a, int variant) {
-  mlp_or_encode<Geo, false>(a->f_in, a->f_out, a->geo, a->tau0, a->taus, a->packed, variant,
-                            a->rows, nullptr, nullptr, a->stw);
+  mlp_or_encode<Geo, false, true>(a->f_in, a->f_out, a->geo, a->tau0, a->taus, a->packed, variant,
+                                  a->rows, nullptr, nullptr, a->stw);
 }
 
 // The step of the MLP-only network; another one is refused.
@@ -529,8 +531,8 @@ __global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
     if (threadIdx.x == 0) raise_status(stw, ST_BLOB);
     return;
   }
-  mlp_or_encode<Geo, false>(f_in, f_out, geo, tau0, taus, packed, variant, rows, nullptr, nullptr,
-                            stw);
+  mlp_or_encode<Geo, false, false>(f_in, f_out, geo, tau0, taus, packed, variant, rows, nullptr,
+                                   nullptr, stw);
 }
 
 // The first launch of a GNN-LBM step, whichever network the image holds: the
@@ -538,14 +540,14 @@ __global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1) gnn_mlp_step_kernel(
 template <class Geo>
 __global__ void __launch_bounds__(128 * LBM_MLP_GROUPS, 1)
     gnn_step_first_kernel(const __grid_constant__ MlpArgs<Geo> a) {
-  dep_sync();  // (the first kernel of a call: the next one may set up)
+  dep_wait();
   if (!blob_ok(a.packed, a.stw)) return;
   const int variant = variant_of(reinterpret_cast<const float*>(a.packed + K::NORM));
   if (variant & VAR_MLP_ONLY)
     mlp_only_step<Geo>(&a, variant);
   else
-    mlp_or_encode<Geo, true>(a.f_in, nullptr, a.geo, 1.0f, nullptr, a.packed, 0, a.rows, a.h0, a.b,
-                             a.stw);
+    mlp_or_encode<Geo, true, true>(a.f_in, nullptr, a.geo, 1.0f, nullptr, a.packed, 0, a.rows, a.h0,
+                                   a.b, a.stw);
 }
 
 template <class Geo>
