@@ -223,4 +223,65 @@ __device__ __forceinline__ void dep_sync() {
   dep_release();
 }
 
+// Reads of what the kernel before may have written.  A kernel launched early
+// runs while that one still does, so neither __ldg nor a const __restrict__
+// pointer may be used for them: both declare the data unchanged for as long as
+// the kernel runs, and such a load may be moved above dep_wait().  ld_prev is a
+// plain load; its address depends on an index or a pointer that went through
+// after_wait(), which stands after dep_wait(), so that it cannot be moved above
+// the wait either.  (Volatile loads keep their order among themselves too: with
+// them the message-passing rounds took 3 % longer, the 64 x 256^2 training step
+// 1 %.)
+template <typename T>
+__device__ __forceinline__ T after_wait(T v) {
+  static_assert(sizeof(T) == 8 || sizeof(T) == 4, "an index or a pointer");
+  if constexpr (sizeof(T) == 8) {
+    uint64_t w = (uint64_t)v;
+    asm volatile("" : "+l"(w) : : "memory");
+    return (T)w;
+  } else {
+    uint32_t w = (uint32_t)v;
+    asm volatile("" : "+r"(w) : : "memory");
+    return (T)w;
+  }
+}
+__device__ __forceinline__ float ld_prev(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_prev(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ unsigned ld_prev(const unsigned* p) {
+  unsigned v;
+  asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_prev(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_prev(const uint4* p) {
+  uint4 v;
+  asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+// The read in a kernel that comes in two instances, of which EARLY alone is
+// launched early: nothing writes the data while the other one runs.
+template <bool EARLY, typename T>
+__device__ __forceinline__ T ld_in(const T* p) {
+  if constexpr (EARLY)
+    return ld_prev(p);
+  else
+    return __ldg(p);
+}
+
 }  // namespace lbmgnn

@@ -83,7 +83,7 @@ static_assert(LBM_PACKED_LAYOUT_VERSION >= 1 && LBM_PACKED_LAYOUT_VERSION <= 9,
 // thread 0 of each CTA raises ST_BLOB and the whole CTA returns before any
 // other access, so nothing is computed from it.
 __device__ __forceinline__ bool blob_ok(const uint8_t* packed, unsigned* stw) {
-  if (__ldg(reinterpret_cast<const unsigned*>(packed + K::MAGIC_SLOT)) == K::MAGIC) return true;
+  if (ld_prev(reinterpret_cast<const unsigned*>(packed + K::MAGIC_SLOT)) == K::MAGIC) return true;
   if (threadIdx.x == 0 && stw) atomicOr(stw, (unsigned)ST_BLOB);
   return false;
 }
@@ -361,7 +361,7 @@ __device__ __forceinline__ float4* chunk4w(float* base, int64_t N, int64_t n, in
 __device__ __forceinline__ void ld_pb32(const __nv_bfloat16* base, int64_t N, int64_t n, int f0,
                                         float* v) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) unpack_bf16x8(__ldg(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
+  for (int c = 0; c < 4; ++c) unpack_bf16x8(ld_prev(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
 }
 __device__ __forceinline__ void st_pb32(__nv_bfloat16* base, int64_t N, int64_t n, int f0,
                                         const float* v) {
@@ -373,10 +373,11 @@ __device__ __forceinline__ void st_ph32(__half* base, int64_t N, int64_t n, int 
   for (int c = 0; c < 4; ++c) *chunk8w(base, N, n, f0 + 8 * c) = pack_h8(v + 8 * c);
 }
 // 32 FP32 values (features f0..f0+31) of node n / their store.
+template <bool EARLY>
 __device__ __forceinline__ void ld_pf32(const float* base, int64_t N, int64_t n, int f0, float* v) {
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const float4 t = __ldg(chunk4(base, N, n, f0 + 4 * c));
+    const float4 t = ld_in<EARLY>(chunk4(base, N, n, f0 + 4 * c));
     v[4 * c] = t.x;
     v[4 * c + 1] = t.y;
     v[4 * c + 2] = t.z;
@@ -390,11 +391,11 @@ __device__ __forceinline__ void st_pf32(float* base, int64_t N, int64_t n, int f
 }
 
 // NF (16 or 32) values versions of the helpers above.
-template <int NF>
+template <int NF, bool EARLY>
 __device__ __forceinline__ void ld_pf(const float* base, int64_t N, int64_t n, int f0, float* v) {
 #pragma unroll
   for (int c = 0; c < NF / 4; ++c) {
-    const float4 t = __ldg(chunk4(base, N, n, f0 + 4 * c));
+    const float4 t = ld_in<EARLY>(chunk4(base, N, n, f0 + 4 * c));
     v[4 * c] = t.x;
     v[4 * c + 1] = t.y;
     v[4 * c + 2] = t.z;
@@ -411,7 +412,7 @@ template <int NF>
 __device__ __forceinline__ void ld_pb(const __nv_bfloat16* base, int64_t N, int64_t n, int f0,
                                       float* v) {
 #pragma unroll
-  for (int c = 0; c < NF / 8; ++c) unpack_bf16x8(__ldg(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
+  for (int c = 0; c < NF / 8; ++c) unpack_bf16x8(ld_prev(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
 }
 template <int NF>
 __device__ __forceinline__ void st_pb(__nv_bfloat16* base, int64_t N, int64_t n, int f0,
@@ -634,10 +635,17 @@ __device__ __forceinline__ uint8_t* smem_align1024(uint8_t* raw) {
 }
 
 // Copies `bytes` (multiple of 16) from global to shared memory with all threads.
+// PREV: the kernel before may have written them (ld_prev).
+template <bool PREV = false>
 __device__ __forceinline__ void copy_g2s(void* dst, const void* src, uint32_t bytes) {
   const uint4* s = reinterpret_cast<const uint4*>(src);
   uint4* d = reinterpret_cast<uint4*>(dst);
-  for (uint32_t i = threadIdx.x; i < bytes / 16; i += blockDim.x) d[i] = __ldg(s + i);
+  for (uint32_t i = threadIdx.x; i < bytes / 16; i += blockDim.x) {
+    if constexpr (PREV)
+      d[i] = ld_prev(s + i);
+    else
+      d[i] = __ldg(s + i);
+  }
 }
 
 // Per-CTA tensor-core context: TMEM base, MMA-completion barrier and phase.

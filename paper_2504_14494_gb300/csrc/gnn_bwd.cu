@@ -41,14 +41,14 @@ __device__ __forceinline__ void st_col(uint8_t* op, int R, int row0, int node, c
 
 // Features f0..f0+NF-1 of node n, BF16 words as they are, into row `row` of an
 // SW128 block.
-template <int NF>
+template <int NF, bool PREV = false>
 __device__ __forceinline__ void copy_row(uint8_t* blk, int row, int f0, const __nv_bfloat16* base,
                                          int64_t N, int64_t n) {
 #pragma unroll
   for (int c = 0; c < NF / 8; ++c) {
     const int chunk = (f0 >> 3) + c;
     *reinterpret_cast<uint4*>(blk + row * 128 + ((chunk ^ (row & 7)) << 4)) =
-        __ldg(chunk8(base, N, n, f0 + 8 * c));
+        ld_in<PREV>(chunk8(base, N, n, f0 + 8 * c));
   }
 }
 
@@ -135,34 +135,33 @@ __device__ __forceinline__ void st_f32x32(float* p, const float* v) {
 // network's time t; d f_pred / d t = ((f - f_eq) + S/2) / t^2.
 template <bool FORCED>
 __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
-    const float* __restrict__ f_pre, const float* __restrict__ y, const float* __restrict__ tgt,
-    Shape s, float tau, const float* __restrict__ taus, float gx0,
-    const float* __restrict__ gxs, const uint8_t* __restrict__ packed,
-    double* __restrict__ lossp, float* __restrict__ dy, float* __restrict__ f_pred,
-    const float* __restrict__ lw, unsigned* stw) {
+    const float* f_pre, const float* y, const float* tgt, Shape s, float tau, const float* taus,
+    float gx0, const float* gxs, const uint8_t* packed, double* __restrict__ lossp,
+    float* __restrict__ dy, float* __restrict__ f_pred, const float* lw, unsigned* stw) {
   dep_sync();
+  packed = after_wait(packed);
   if (!blob_ok(packed, stw)) {  // no loss from an invalid image: NaN
     if (threadIdx.x == 0) lossp[blockIdx.x] = __longlong_as_double(0x7ff8000000000000LL);
     return;
   }
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
-  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = after_wait((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const bool on = n < N;
   const int64_t nn = on ? n : N - 1;
   const float sdf = reinterpret_cast<const float*>(packed + K::NORM)[24];
   const int variant = variant_of(reinterpret_cast<const float*>(packed + K::NORM));
   float fv[Q], yv[NOUT];
 #pragma unroll
-  for (int q = 0; q < Q; ++q) fv[q] = __ldg(f_pre + q * s.ps + nn);
+  for (int q = 0; q < Q; ++q) fv[q] = ld_prev(f_pre + q * s.ps + nn);
 #pragma unroll
-  for (int o = 0; o < NOUT; ++o) yv[o] = __ldg(y + o * N + nn);
+  for (int o = 0; o < NOUT; ++o) yv[o] = ld_prev(y + o * N + nn);
   const int64_t b = nn / ((int64_t)s.nx * s.ny);
-  const float t = taus ? __ldg(taus + b) : tau;
-  const float wb = lw ? __ldg(lw + b) : 1.0f;  // per-instance loss weight (1: Eq. 4)
+  const float t = taus ? ld_prev(taus + b) : tau;
+  const float wb = lw ? ld_prev(lw + b) : 1.0f;  // per-instance loss weight (1: Eq. 4)
   Moments m = moments9(fv);
   float gx = 0.0f;
   if constexpr (FORCED) {
-    gx = gxs ? __ldg(gxs + b) : gx0;
+    gx = gxs ? ld_prev(gxs + b) : gx0;
     m.ux += 0.5f * gx / m.rho;
   }
   const float usq15 = 1.5f * (m.ux * m.ux + m.uy * m.uy);
@@ -187,7 +186,7 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
       fp += (1.0f - 0.5f * inv) * src;
       dt += 0.5f * src;
     }
-    const float r = fp - __ldg(tgt + q * s.ps + nn);
+    const float r = fp - ld_prev(tgt + q * s.ps + nn);
     rr[q] = r;
     // wb r^2 as an FP32 pair: the rounding errors of both products are exact
     const float r2 = r * r, w2 = wb * r2;
@@ -238,13 +237,13 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
 __global__ void __launch_bounds__(256) gnn_collide_adjoint_kernel(
     const float* __restrict__ f_pre, const float* __restrict__ y,
     const float* __restrict__ f_post, const float* __restrict__ tgt,
-    const float* __restrict__ g_in, Shape s, float tau, const float* __restrict__ taus,
+    const float* g_in, Shape s, float tau, const float* __restrict__ taus,
     const uint8_t* __restrict__ packed, float scale, float* __restrict__ dy,
     float* __restrict__ dfd, unsigned* stw) {
   dep_sync();
   if (!blob_ok(packed, stw)) return;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
-  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = after_wait((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   if (n >= N) return;
   const float* nrm = reinterpret_cast<const float*>(packed + K::NORM);
   const float sdf = nrm[24];
@@ -254,7 +253,7 @@ __global__ void __launch_bounds__(256) gnn_collide_adjoint_kernel(
   for (int q = 0; q < Q; ++q) {
     fv[q] = __ldg(f_pre + q * s.ps + n);
     const float r = __ldg(f_post + q * s.ps + n) - __ldg(tgt + q * s.ps + n);
-    g[q] = (g_in ? __ldg(g_in + q * s.ps + n) : 0.0f) + scale * r;
+    g[q] = (g_in ? ld_prev(g_in + q * s.ps + n) : 0.0f) + scale * r;
     gp[q] = g[q];
   }
   const float y0 = __ldg(y + n);
@@ -308,14 +307,14 @@ __global__ void __launch_bounds__(256) stream_adjoint_sum_kernel(
 // Sum of the per-block squared errors, divided by 9 N (deterministic order).
 // One block: 1,024 threads with 8 loads in flight each (34 us for 16,384
 // values with 256 threads and one load at a time).
-__global__ void __launch_bounds__(1024) loss_finish_kernel(const double* __restrict__ lossp,
-                                                           int nblk, double count,
+__global__ void __launch_bounds__(1024) loss_finish_kernel(const double* lossp, int nblk,
+                                                           double count,
                                                            double* __restrict__ loss) {
   dep_sync();
   __shared__ double red[32];
   double acc = 0.0;
 #pragma unroll 8
-  for (int i = threadIdx.x; i < nblk; i += 1024) acc += __ldg(lossp + i);
+  for (int i = after_wait((int)threadIdx.x); i < nblk; i += 1024) acc += ld_prev(lossp + i);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -341,15 +340,16 @@ constexpr uint32_t XT = 0, ONE = 32768, H2 = 36864, WHF = 53248, DYS = 55808, SH
 #define LBM_HB_CTAS 2  // resident CTAs per SM
 #endif
 __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
-    const float* __restrict__ dy, const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh,
-    float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
+    const float* dy, const __nv_bfloat16* h2, float* __restrict__ dh, float* __restrict__ G,
+    Shape s, const uint8_t* packed, unsigned* stw) {
   dep_wait();  // before the weights: as a call's first kernel it may follow their pack
+  packed = after_wait(packed);
   if (!blob_ok(packed, stw)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_align1024(smem_raw);
   TcShared* sh = reinterpret_cast<TcShared*>(sm + hb::SH);
   zero_smem(sm, hb::H2);
-  copy_g2s(sm + hb::WHF, packed + K::WHF, 2560);
+  copy_g2s<true>(sm + hb::WHF, packed + K::WHF, 2560);
   __syncthreads();
   ones_row(sm + hb::ONE, 16, 0);
   TcCtx tc;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   const int64_t ntiles = (N + TILE - 1) / TILE;
   bool first = true, ok = true;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int64_t tile = after_wait((int64_t)blockIdx.x); tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
@@ -377,12 +377,12 @@ __global__ void __launch_bounds__(256, LBM_HB_CTAS) gnn_head_bwd_kernel(
       float d[NOUT];
 #pragma unroll
       for (int o = 0; o < NOUT; ++o) {
-        d[o] = on ? __ldg(dy + o * N + nn) : 0.0f;
+        d[o] = on ? ld_prev(dy + o * N + nn) : 0.0f;
         dys[node * NOUT + o] = d[o];
       }
       st_col<NOUT>(XT, 128, 0, node, d);
     }
-    copy_row<32>(H2, node, f0, h2, N, nn);
+    copy_row<32, true>(H2, node, f0, h2, N, nn);
     __syncthreads();
     float dv[32];
 #pragma unroll
@@ -440,9 +440,10 @@ constexpr uint32_t HA = 0, DZ = 32768, WN = 49152, BN = 65536, DBR = 65792, SH =
 #define LBM_RB1_CTAS 2  // resident CTAs per SM
 #endif
 
+template <bool EARLY>
 __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
     const __nv_bfloat16* __restrict__ h_in, const __nv_bfloat16* __restrict__ a_in,
-    const float* __restrict__ dh_out, float* __restrict__ dh_part, float* __restrict__ da,
+    const float* dh_out, float* __restrict__ dh_part, float* __restrict__ da,
     int round, float* __restrict__ G, Shape s, const uint8_t* __restrict__ packed, unsigned* stw) {
   if (!blob_ok(packed, stw)) return dep_sync();
   extern __shared__ uint8_t smem_raw[];
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
   float dbacc = 0.0f;  // lane l: running sum of dz[f0 + l] over this warp's nodes
   bool first = true, ok = true;
   dep_sync();
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int64_t tile = EARLY ? after_wait((int64_t)blockIdx.x) : blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
     {
       float dz[32], dho[32];
       tmem_ld32(lb + f0, dz);
-      ld_pf32(dh_out, N, nn, f0, dho);
+      ld_pf32<EARLY>(dh_out, N, nn, f0, dho);
       act_and_grad(dz, bn + f0, 32, false, nullptr, dz);  // GELU'(z_n), packed pairs
 #pragma unroll
       for (int c = 0; c < 32; ++c) dz[c] = (on && !mlp_only) ? dho[c] * dz[c] : 0.0f;
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(256, LBM_RB1_CTAS) gnn_round_bwd1_kernel(
     {
       float d[32], dho[32];
       tmem_ld32(lb + f0, d);           // warp-collective: every lane takes part
-      ld_pf32(dh_out, N, nn, f0, dho);  // again (an L2 hit): fewer values live across the MMA
+      ld_pf32<EARLY>(dh_out, N, nn, f0, dho);  // again (an L2 hit): fewer values live across the MMA
 #pragma unroll
       for (int c = 0; c < 32; ++c) d[c] += dho[c];
       if (on) st_pf32(dh_part, N, n, f0, d);
@@ -565,10 +566,10 @@ constexpr uint32_t DAB = 0, H = 32768, ONE = 49152, WABT = 53248, CK = 69632, CK
 // training step 11.18 -> 10.85 ms, a step of few tiles 37 -> 31 us per launch.
 // dA and dB direction by direction in one loop (two independent chains)
 // instead of one after the other: 10.85 -> 10.38 ms.
-template <bool WALLS>
+template <bool WALLS, bool EARLY>
 __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
-    const __half* __restrict__ ab, const float* __restrict__ da,
-    const float* __restrict__ dh_part, const __nv_bfloat16* __restrict__ h_in,
+    const __half* __restrict__ ab, const float* da, const float* dh_part,
+    const __nv_bfloat16* __restrict__ h_in,
     float* __restrict__ dh_in, int round, float* __restrict__ G, Shape s,
     const uint8_t* __restrict__ packed, unsigned* stw) {
   if (!blob_ok(packed, stw)) return dep_sync();
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
   const int64_t ntiles = (N + TILE - 1) / TILE;
   bool first = true, ok = true;
   dep_sync();
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int64_t tile = EARLY ? after_wait((int64_t)blockIdx.x) : blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
@@ -643,7 +644,7 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
         ai[kk][0] = __ldg(chunk8(ab, N, i, c0));
         ai[kk][1] = __ldg(chunk8(ab, N, i, c0 + 8));
 #pragma unroll
-        for (int t4 = 0; t4 < 4; ++t4) di[kk][t4] = __ldg(chunk4(da, N, i, c0 + 4 * t4));
+        for (int t4 = 0; t4 < 4; ++t4) di[kk][t4] = ld_in<EARLY>(chunk4(da, N, i, c0 + 4 * t4));
       }
 #pragma unroll
       for (int kk = 0; kk < GROUP; ++kk) {
@@ -675,7 +676,7 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
       float gA[16], v[32];  // v = [dc_x | dc_y] of this node
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float4 t = __ldg(chunk4(da, N, nn, c0 + 4 * i));
+        const float4 t = ld_in<EARLY>(chunk4(da, N, nn, c0 + 4 * i));
         const float dd[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {  // the factor 1/2 of 2 GELU' is applied here
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(512, 1) gnn_round_bwd2_kernel(
     float d[NF], dp[NF];
     tmem_ld<NF>(lb + f0, d);
     if (on) {
-      ld_pf<NF>(dh_part, N, n, f0, dp);
+      ld_pf<NF, EARLY>(dh_part, N, n, f0, dp);
 #pragma unroll
       for (int c = 0; c < NF; ++c) d[c] += dp[c];
       st_pf<NF>(dh_in, N, n, f0, d);
@@ -775,8 +776,9 @@ constexpr uint32_t G1 = 0, DZ = 16384, XH = 49152, W2 = 53248, W1F = 61440, B1 =
 // The channel's velocity feature is (sum f e + F/2)/rho with F = (fx, 0)
 // (fxs[b] per lattice when set; fx = 0 and fxs NULL elsewhere); its
 // derivative w.r.t. f_i is (e_i - u)/rho with that u.
+template <bool EARLY>
 __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
-    const float* __restrict__ f_pre, const float* __restrict__ dh0, float* __restrict__ df,
+    const float* __restrict__ f_pre, const float* dh0, float* __restrict__ df,
     float* __restrict__ G, Shape s, float fx, const float* __restrict__ fxs,
     const uint8_t* __restrict__ packed, unsigned* stw) {
   if (!blob_ok(packed, stw)) return dep_sync();
@@ -810,7 +812,7 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
   const int64_t ntiles = (N + TILE - 1) / TILE;
   bool first = true, ok = true;
   dep_sync();
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int64_t tile = EARLY ? after_wait((int64_t)blockIdx.x) : blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n = tile * TILE + node;
     const bool on = n < N;
     const int64_t nn = on ? n : N - 1;
@@ -859,7 +861,7 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
     {
       float z2[32], g0[32];
       tmem_ld32(lb + f0, z2);
-      ld_pf32(dh0, N, nn, f0, g0);
+      ld_pf32<EARLY>(dh0, N, nn, f0, g0);
       act_and_grad(z2, b2 + f0, 32, relu, nullptr, d);
 #pragma unroll
       for (int c = 0; c < 32; ++c) d[c] = on ? g0[c] * d[c] : 0.0f;
@@ -947,12 +949,11 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
 struct GradRows {
   int enc, edge, node, head;
 };
-__global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict__ G,
-                                                         GradRows rows, float* __restrict__ grad,
-                                                         bool accumulate,
+__global__ void __launch_bounds__(64) grad_reduce_kernel(const float* G, GradRows rows,
+                                                         float* __restrict__ grad, bool accumulate,
                                                          const uint8_t* __restrict__ packed) {
   dep_sync();
-  const int p = blockIdx.x * 64 + threadIdx.x;
+  const int p = after_wait((int)(blockIdx.x * 64 + threadIdx.x));
   if (p >= P::TRAINABLE) return;
   int n = rows.enc;
   if (p >= P::HEAD_W)
@@ -967,7 +968,7 @@ __global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict
     float v[BATCH];
 #pragma unroll
     for (int i = 0; i < BATCH; ++i)
-      v[i] = r0 + i < n ? __ldg(G + (int64_t)(r0 + i) * P::TRAINABLE + p) : 0.0f;
+      v[i] = r0 + i < n ? ld_prev(G + (int64_t)(r0 + i) * P::TRAINABLE + p) : 0.0f;
 #pragma unroll
     for (int i = 0; i < BATCH; ++i) acc += v[i];
   }
@@ -975,13 +976,13 @@ __global__ void __launch_bounds__(64) grad_reduce_kernel(const float* __restrict
 }
 
 // AdamW (decoupled weight decay) on the trainable prefix.
-__global__ void adamw_kernel(float* __restrict__ theta, const float* __restrict__ g,
+__global__ void adamw_kernel(float* __restrict__ theta, const float* g,
                              float* __restrict__ m, float* __restrict__ v, float lr, float wd,
                              float b1, float b2, float eps, float bc1, float bc2) {
   dep_sync();
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = after_wait((int)(blockIdx.x * blockDim.x + threadIdx.x));
   if (p >= P::TRAINABLE) return;
-  const float gp = g[p];
+  const float gp = ld_prev(g + p);
   const float mp = b1 * m[p] + (1.0f - b1) * gp;
   const float vp = b2 * v[p] + (1.0f - b2) * gp * gp;
   m[p] = mp;
@@ -1078,14 +1079,18 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
   for (int r = 1; r >= 0; --r) {
     {
       const uint32_t bytes = rb1::BYTES + 1024;
-      if ((e = set_smem(gnn_round_bwd1_kernel, bytes)) != cudaSuccess) return e;
-      if ((e = launch_after(early, gnn_round_bwd1_kernel, rows.node, 256, bytes, st, hs[r], as[r], bl.dh[0],
+      auto* kern = early ? gnn_round_bwd1_kernel<true> : gnn_round_bwd1_kernel<false>;
+      if ((e = set_smem(kern, bytes)) != cudaSuccess) return e;
+      if ((e = launch_after(early, kern, rows.node, 256, bytes, st, hs[r], as[r], bl.dh[0],
                             bl.dh[1], bl.da, r, bl.G, s, packed, stw)) != cudaSuccess)
         return e;
     }
     {
       const uint32_t bytes = rb2::BYTES + 1024;
-      auto* kern = bl.walls ? gnn_round_bwd2_kernel<true> : gnn_round_bwd2_kernel<false>;
+      auto* kern = bl.walls ? (early ? gnn_round_bwd2_kernel<true, true>
+                                     : gnn_round_bwd2_kernel<true, false>)
+                            : (early ? gnn_round_bwd2_kernel<false, true>
+                                     : gnn_round_bwd2_kernel<false, false>);
       if ((e = set_smem(kern, bytes)) != cudaSuccess) return e;
       if ((e = launch_after(early, kern, rows.edge, 512, bytes, st, abs_[r], bl.da, bl.dh[1],
                             hs[r], bl.dh[0], r, bl.G, s, packed, stw)) != cudaSuccess)
@@ -1094,8 +1099,9 @@ cudaError_t launch_gnn_backward(const BackwardLaunch& bl, const Shape& s, const 
   }
   {
     const uint32_t bytes = eb::BYTES + 1024;
-    if ((e = set_smem(gnn_encode_bwd_kernel, bytes)) != cudaSuccess) return e;
-    if ((e = launch_after(early, gnn_encode_bwd_kernel, rows.enc, 256, bytes, st, bl.f_pre, bl.dh[0], bl.df,
+    auto* kern = early ? gnn_encode_bwd_kernel<true> : gnn_encode_bwd_kernel<false>;
+    if ((e = set_smem(kern, bytes)) != cudaSuccess) return e;
+    if ((e = launch_after(early, kern, rows.enc, 256, bytes, st, bl.f_pre, bl.dh[0], bl.df,
                           bl.G, s, bl.fx, bl.fxs, packed, stw)) != cudaSuccess)
       return e;
   }

@@ -31,9 +31,16 @@ __device__ __forceinline__ void put_sw(uint8_t* blk, int row, int k, float v) {
   *reinterpret_cast<__nv_bfloat16*>(blk + sw128_off(row, k)) = __float2bfloat16_rn(v);
 }
 
-__global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict__ out,
-                                unsigned* stw) {
+// The parameter vector: the kernel before (AdamW) may have written it.
+struct PrevParams {
+  const float* p;
+  __device__ __forceinline__ float operator[](int i) const { return ld_prev(p + i); }
+  __device__ __forceinline__ PrevParams operator+(int i) const { return {p + i}; }
+};
+
+__global__ void gnn_pack_kernel(const float* params, uint8_t* __restrict__ out, unsigned* stw) {
   dep_sync();
+  const PrevParams p{after_wait(params)};
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
   float* w1f = reinterpret_cast<float*>(out + K::W1F);
@@ -91,10 +98,10 @@ __global__ void gnn_pack_kernel(const float* __restrict__ p, uint8_t* __restrict
     put_sw(out + K::W1X, o, k, w);
   }
   for (int r = 0; r < 2; ++r) {
-    const float* pr = p + P::ROUND0 + r * P::ROUND_SIZE;
+    const PrevParams pr = p + P::ROUND0 + r * P::ROUND_SIZE;
     uint8_t* kr = out + K::round_base(r);
-    const float* we = pr + P::EDGE_W;  // [64][130]
-    const float* wn = pr + P::NODE_W;  // [64][128]
+    const PrevParams we = pr + P::EDGE_W;  // [64][130]
+    const PrevParams wn = pr + P::NODE_W;  // [64][128]
     for (int e = at(3 + r); e < HID * HID; e += nth) {
       const int o = e / HID, i = e % HID;
       const float wa = we[o * 130 + i], wb = we[o * 130 + HID + i];
@@ -368,7 +375,8 @@ __global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_k
   const int64_t N = geo.count();
   const int64_t base = geo.base(), ps = geo.ps();
   const int64_t ntiles = (N + TILE - 1) / TILE;
-  const int64_t first = (int64_t)blockIdx.x * NG + grp, stride = (int64_t)gridDim.x * NG;
+  const int64_t stride = (int64_t)gridDim.x * NG;
+  int64_t first = (int64_t)blockIdx.x * NG + grp;
   const int variant = variant_of(nrm);
   const bool mlp_only = variant & VAR_MLP_ONLY;
   const __nv_bfloat16* h_src = (mlp_only && ra.h_skip) ? ra.h_skip : ra.h_in;
@@ -378,15 +386,19 @@ __global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_k
     return true;
   };
 
+  // The inputs are the kernel before's outputs; with four threads per node this
+  // one is launched early (round_launch).
+  constexpr bool EARLY = TPN == 4;
   // raw BF16 h (features f0.. of node `t * TILE + node`) of tile t
   uint4 hnext[FPT / 8];
   auto load_h = [&](int64_t t) {
     const int64_t m = t * TILE + node;
     const int64_t mm = m < N ? m : N - 1;
 #pragma unroll
-    for (int c = 0; c < FPT / 8; ++c) hnext[c] = __ldg(chunk8(h_src, N, mm, f0 + 8 * c));
+    for (int c = 0; c < FPT / 8; ++c) hnext[c] = ld_in<EARLY>(chunk8(h_src, N, mm, f0 + 8 * c));
   };
   dep_sync();
+  if constexpr (EARLY) first = after_wait(first);
   if (AH && first < ntiles) load_h(first);
 
   for (int64_t tile = first; tile < ntiles; tile += stride) {
@@ -409,7 +421,9 @@ __global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_k
 #pragma unroll
       for (int s0 = 0; s0 < FPT; s0 += SL) {
         float h[SL];
-        ld_pb<SL>(h_src, N, nn, f0 + s0, h);
+#pragma unroll
+        for (int c = 0; c < SL / 8; ++c)
+          unpack_bf16x8(ld_in<EARLY>(chunk8(h_src, N, nn, f0 + s0 + 8 * c)), h + 8 * c);
         st_row<SL>(H, node, f0 + s0, h);
       }
     }
@@ -433,8 +447,8 @@ __global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_k
 #pragma unroll
         for (int c = 0; c < 8; ++c) aw[c] = h2_as_u32(__floats2half2_rn(av[2 * c], av[2 * c + 1]));
       } else {
-        const uint4 a0 = __ldg(chunk8(ra.ab_in, N, nn, c0));
-        const uint4 a1 = __ldg(chunk8(ra.ab_in, N, nn, c0 + 8));
+        const uint4 a0 = ld_in<EARLY>(chunk8(ra.ab_in, N, nn, c0));
+        const uint4 a1 = ld_in<EARLY>(chunk8(ra.ab_in, N, nn, c0 + 8));
         aw[0] = a0.x, aw[1] = a0.y, aw[2] = a0.z, aw[3] = a0.w;
         aw[4] = a1.x, aw[5] = a1.y, aw[6] = a1.z, aw[7] = a1.w;
       }
@@ -451,8 +465,8 @@ __global__ void __launch_bounds__(128 * TPN * NG, round_ctas<TPN>()) gnn_round_k
         for (int k = 0; k < LBM_NBR_GROUP; ++k) {
           const int64_t j = checked(geo_nbr(p, ex(g + k + 1), ey(g + k + 1)) - base, 0, N, stw);
           constexpr int BOFF = AH ? 0 : HID;  // B's first feature in ab_in
-          braw[k][0] = __ldg(chunk8(ra.ab_in, N, j, BOFF + c0));
-          braw[k][1] = __ldg(chunk8(ra.ab_in, N, j, BOFF + c0 + 8));
+          braw[k][0] = ld_in<EARLY>(chunk8(ra.ab_in, N, j, BOFF + c0));
+          braw[k][1] = ld_in<EARLY>(chunk8(ra.ab_in, N, j, BOFF + c0 + 8));
         }
 #pragma unroll
         for (int k = 0; k < LBM_NBR_GROUP; ++k) {

@@ -1,6 +1,8 @@
 """Ordering rules of the device code that no run can show to be kept, checked
 on the source (csrc/): a kernel that lets its successor start early
-(dep_release, common.cuh) allocates its tensor memory first."""
+(dep_release, common.cuh) allocates its tensor memory first, and a kernel that
+starts early reads its predecessor's outputs by loads that stay where they are
+(ld_prev)."""
 import glob
 import os
 import re
@@ -58,3 +60,52 @@ def test_tensor_memory_is_allocated_before_the_successor_is_released():
     # every kernel of the early-launched calls that uses tensor memory
     assert {"gnn_encode_kernel", "gnn_round_kernel", "gnn_head_bwd_kernel", "gnn_round_bwd1_kernel",
             "gnn_round_bwd2_kernel", "gnn_encode_bwd_kernel", "mlp_or_encode"} <= seen
+
+
+# Buffers that the kernel before may still be writing when a kernel launched
+# early starts (None: it may be the first kernel of a call, so all of them).
+PREVIOUS = {
+    "gnn_pack_kernel": None, "adamw_kernel": None, "gnn_head_bwd_kernel": None,
+    "gnn_collide_loss_kernel": None,
+    "gnn_round_kernel": ["h_src", "ra.ab_in"],      # the encoder's or the round's before
+    "loss_finish_kernel": ["lossp"],
+    "gnn_collide_adjoint_kernel": ["g_in"],         # stream_adjoint_sum_kernel's
+    "stream_adjoint_sum_kernel": [],                # follows grad_reduce_kernel, reads older outputs
+    "gnn_round_bwd1_kernel": ["dh_out"],            # the head's or the edge backward's
+    "gnn_round_bwd2_kernel": ["da", "dh_part"],
+    "gnn_encode_bwd_kernel": ["dh0"],
+    "grad_reduce_kernel": ["G"],
+}
+LOADERS = ("ld_pf", "ld_pf32", "copy_row", "blob_ok")
+
+
+def test_outputs_of_the_kernel_before_are_not_declared_unchanged():
+    """What the kernel before an early-launched one writes is read at addresses
+    formed after the wait, without __ldg and without a const __restrict__
+    pointer (both promise that the data does not change while the kernel
+    runs)."""
+    funcs = functions()
+    for name in LOADERS:
+        assert "__ldg(" not in funcs[name][1], name
+    early = set()
+    for path in glob.glob(os.path.join(CSRC, "*.cu")):
+        src = _strip(open(path).read())
+        early |= set(re.findall(r"launch_after\(\s*[^,()]*(?:==[^,()]*)?,\s*(?:kern\b|(\w+))", src))
+    # (those launched through `kern`, by the size of the call)
+    early = {n for n in early if n} | {"gnn_round_bwd1_kernel", "gnn_round_bwd2_kernel",
+                                       "gnn_encode_bwd_kernel"}
+    assert early == set(PREVIOUS)
+    pointer = re.compile(r"const\s+\w+\s*\*\s*(__restrict__\s+)?(\w+)")
+    for name, buffers in PREVIOUS.items():
+        params, body = funcs[name]
+        if buffers is None:
+            assert "__ldg(" not in body and "copy_g2s(" not in body, name
+            assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", params), name
+            buffers = [m.group(2) for m in pointer.finditer(params)]
+        for b in buffers:
+            assert not re.search(r"__ldg\((?:chunk[48]\()?" + re.escape(b) + r"\b", body), (name, b)
+            assert b not in [m.group(2) for m in pointer.finditer(params) if m.group(1)], (name, b)
+        if buffers:
+            wait = max(m.end() for m in re.finditer(r"(?<!return )\bdep_(?:sync|wait)\(\)", body))
+            taken = [m.start() for m in re.finditer(r"\bafter_wait\(", body)]
+            assert taken and min(taken) > wait, name
