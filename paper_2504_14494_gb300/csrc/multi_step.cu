@@ -66,8 +66,9 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
 // Between two steps the CTAs of a cluster exchange their edge rows: each edge
 // node's three outgoing populations go to the neighbour's halo row by st.async,
 // which counts their bytes on an mbarrier there; the threads of the edge rows
-// wait for the halo's bytes, the others only for their own CTA.  (A cluster
-// barrier per step in its place: 0.75 us a step at 64^2.)  There is one
+// wait for the halo's bytes (an acquire at cluster scope), the others only for
+// their own CTA.  (A cluster barrier per step in its place: 0.75 us a step at
+// 64^2.)  There is one
 // mbarrier per buffer: a CTA cannot start step n + 2 before its neighbours have
 // sent step n + 1, so a neighbour is at most one step ahead.
 struct ResidentArgs {
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, un
         // the halo of this step's buffer (step 0: loaded above)
         if (step > 0 && (first_row[k] || last_row[k])) {
           const int h = step & 1;  // filled during step - 1
-          if (!mbar_wait(&bar[h], ((step - 1) >> 1) & 1)) lost = true;
+          if (!mbar_wait<true>(&bar[h], ((step - 1) >> 1) & 1)) lost = true;
           if (k == 0 && threadIdx.x == 0) expect_bytes(&bar[h], halo_bytes);  // for step + 2
         }
       }

@@ -2,7 +2,8 @@
 on the source (csrc/): a kernel that lets its successor start early
 (dep_release, common.cuh) allocates its tensor memory first, and a kernel that
 starts early reads its predecessor's outputs by loads that stay where they are
-(ld_prev)."""
+(ld_prev); a wait for what another CTA of a cluster sends acquires at cluster
+scope."""
 import glob
 import os
 import re
@@ -109,3 +110,15 @@ def test_outputs_of_the_kernel_before_are_not_declared_unchanged():
             wait = max(m.end() for m in re.finditer(r"(?<!return )\bdep_(?:sync|wait)\(\)", body))
             taken = [m.start() for m in re.finditer(r"\bafter_wait\(", body)]
             assert taken and min(taken) > wait, name
+
+
+def test_waits_for_another_cta_acquire_at_cluster_scope():
+    senders = 0
+    for name, (_, body) in functions().items():
+        if re.search(r"\bst_async\(", body) and name != "st_async":
+            senders += 1
+            assert not re.search(r"\bmbar_(?:try_)?wait(?:_sleep)?(?:<false>)?\(", body), name
+            assert "mbar_wait<true>(" in body, name
+    assert senders == 1  # the resident multi-step kernel
+    body = functions()["mbar_try_wait_sleep"][1]
+    assert "try_wait.parity.acquire.cluster." in body[:body.index("else")]
