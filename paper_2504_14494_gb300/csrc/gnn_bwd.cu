@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
   const float teff = t * tau_adj_of(yv[0], variant);
   const float inv = 1.0f / teff;
   const float scale = 2.0f * wb / (9.0f * (float)N);
-  DF ls{0.0f, 0.0f};
+  float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;  // sum of r^2, unevaluated
   float dta = 0.0f, dyv[NOUT], d[Q], g[Q], rr[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) d[q] = sdf * yv[1 + q];
@@ -188,13 +188,31 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
     }
     const float r = fp - ld_prev(tgt + q * s.ps + nn);
     rr[q] = r;
-    // wb r^2 as an FP32 pair: the rounding errors of both products are exact
-    const float r2 = r * r, w2 = wb * r2;
-    df_add(ls, w2);
-    ls.lo += fmaf(wb, r2, -w2) + wb * fmaf(r, r, -r2);
+    // r^2 = r2 + fma(r, r, -r2) exactly; the first two sums are error-free
+    const float r2 = __fmul_rn(r, r);
+    float e, f;
+    two_sum(s0, r2, s0, e);
+    two_sum(s1, e, s1, e);
+    two_sum(s1, __fmaf_rn(r, r, -r2), s1, f);
+    s2 = __fadd_rn(s2, __fadd_rn(e, f));
     g[q] = scale * r;  // dL/df*
     dta += g[q] * dt;
     if (on && f_pred) f_pred[q * s.ps + n] = fp;
+  }
+  // The squared error goes on in FP64.  The node's sum S of r^2 was carried in
+  // three FP32 words: s0 and s1 take error-free sums, |s1| <= 18 2^-24 S,
+  // |s2| <= 18 2^-24 |s1|, and the 18 additions into s2 round, which is below
+  // 2^-59 S in all; with the addition and the weight's product here the node's
+  // value is within 2.1 2^-53.  Nine FP64 products and sums, within 10 2^-53,
+  // bound the call (4.2 M nodes, with the finish: 311 us against 169); they are
+  // used where r^2 leaves the range in which its rounding error is an FP32
+  // number.
+  double lp = (double)s0 + ((double)s1 + (double)s2);
+  if (lw) lp *= (double)wb;
+  if (!(s0 >= 1e-25f && s0 < 1e30f)) {
+    lp = 0.0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) lp += (double)wb * (double)rr[q] * (double)rr[q];
   }
   // Delta f = s_df P y_1..9 with P the (symmetric) projection, or P = I
   if (variant & VAR_CONSERVATIVE) conserve9(g);
@@ -204,15 +222,6 @@ __global__ void __launch_bounds__(256) gnn_collide_loss_kernel(
   if (on && dy) {
 #pragma unroll
     for (int o = 0; o < NOUT; ++o) dy[o * N + n] = dyv[o];
-  }
-  // block reduction of the squared error: the node's sum was carried in FP32
-  // pairs (about 2^-46 relative; nine FP64 products per node bound the kernel,
-  // 277 us for 4.2 M nodes), in FP64 where it leaves their range
-  double lp = (double)ls.hi + (double)ls.lo;
-  if (!(ls.hi >= 1e-25f && ls.hi < 1e30f)) {
-    lp = 0.0;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) lp += (double)wb * (double)rr[q] * (double)rr[q];
   }
   if (!on) lp = 0.0;
   __shared__ double red[8];
