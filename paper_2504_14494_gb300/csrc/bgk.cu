@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(128) bgk_step_x4(const float* __restrict__ fin
     }
   }
   if constexpr (TOTALS) {
-    NodeTotals t;
+    NodeTotals<> t;
     if (on) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) t.add(f[j]);
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256) bgk_step_any(const float* __restrict__ fi
     for (int q = 0; q < Q; ++q) fout[q * s.ps + nn] = f[q];
   }
   if constexpr (TOTALS) {
-    NodeTotals t;
+    NodeTotals<> t;
     if (on) t.add(f);
     if (t.bad) raise_status(stw, ST_NONFINITE);
     t.flush<256>(totals);
@@ -162,9 +162,11 @@ __global__ void __launch_bounds__(256) bgk_step_any(const float* __restrict__ fi
 }
 
 // ---------------------------------------------------------------------------
-// Moments of a stored state and FP64 totals.  A thread takes several nodes: a
-// block per 256 nodes ended in 5 atomics on the same 5 words each, which bound
-// the kernel (1.6 M nodes: 43 us).
+// Moments of a stored state and FP64 totals.  A thread takes several nodes, 64
+// at most (the bound of a thread's sums, common.cuh): a block per 256 nodes
+// ended in 5 atomics on the same 5 words each, which bound the kernel (totals
+// of 1.6 M nodes: 49 us, now 25; of 4096^2: 441, now 173; 166 with two words
+// per sum).
 __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ f, Shape s,
                                                       float* __restrict__ rho,
                                                       float* __restrict__ ux,
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ 
                                                       double* __restrict__ totals, unsigned* stw) {
   dep_sync();
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
-  NodeTotals t;
+  NodeTotals<TF> t;
   for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N;
        n += (int64_t)gridDim.x * blockDim.x) {
     float v[Q];
@@ -258,8 +260,9 @@ cudaError_t launch_moments(const float* f, const Shape& s, float* rho, float* ux
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   unsigned* stw = status_word();
   if (totals && !stw) return cudaErrorInvalidDevice;
-  // 1,216 blocks (8 for each of 152 SMs) or fewer
-  const unsigned blocks = (unsigned)std::min<int64_t>((N + 255) / 256, 1216);
+  // 8 blocks per SM, more where a thread would take more than 64 nodes
+  const int64_t few = std::max<int64_t>(8 * std::max(1, sm_count()), (N + 64 * 256 - 1) / (64 * 256));
+  const unsigned blocks = (unsigned)std::min<int64_t>((N + 255) / 256, few);
   moments_kernel<<<blocks, 256, 0, st>>>(f, s, rho, ux, uy, totals, stw);
   return cudaGetLastError();
 }

@@ -96,6 +96,7 @@ __device__ __forceinline__ void bgk_collide(float (&f)[Q], float omega) {
 // renormalised by another TwoSum once per node.  About 2^-46 relative error
 // per node; FP64 arithmetic is used once per warp.
 struct DF {
+  static constexpr bool kPair = true;
   float hi, lo;
 };
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -126,11 +127,46 @@ __device__ __forceinline__ DF df_shfl_xor(const DF& a, int o) {
   return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
 
+// The sum of a thread that takes many nodes, unevaluated s0 + s1 + s2: s0 and s1
+// take error-free sums, s2 collects what s1 rounds off, so that the error does
+// not grow with the nodes as that of a DF does (54 equal nodes: up to 2^-46).
+// For up to 64 nodes of one sign |s1| <= 2^-17 of the sum, |s2| <= 2^-34 and its
+// rounding errors 2^-51.
+struct TF {
+  static constexpr bool kPair = false;
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+  __device__ __forceinline__ void add(float hi) {
+    float e, g;
+    two_sum(s0, hi, s0, e);
+    two_sum(s1, e, s1, g);
+    s2 = __fadd_rn(s2, g);
+  }
+  __device__ __forceinline__ void add(const DF& x) {
+    float g;
+    two_sum(s1, x.lo, s1, g);
+    s2 = __fadd_rn(s2, g);
+    add(x.hi);
+  }
+  __device__ __forceinline__ DF pair() const {  // within 2^-48
+    DF a;
+    two_sum(s0, s1, a.hi, a.lo);
+    a.lo = __fadd_rn(a.lo, s2);
+    df_norm(a);
+    return a;
+  }
+};
+
+__device__ __forceinline__ void df_add(TF& a, const DF& b) { a.add(b); }
+__device__ __forceinline__ DF as_pair(const DF& a) { return a; }
+__device__ __forceinline__ DF as_pair(const TF& a) { return a.pair(); }
+
 // Per-thread totals of stored nodes: mass sum f_i, momentum sum f_i e_i,
 // kinetic energy sum |j|^2 / (2 rho), and the count of nodes holding a
 // non-finite population (excluded from the sums).
+// Sum: DF for a few nodes per thread, TF for many.
+template <class Sum = DF>
 struct NodeTotals {
-  DF m{0.f, 0.f}, px{0.f, 0.f}, py{0.f, 0.f}, e{0.f, 0.f};
+  Sum sm{}, spx{}, spy{}, se{};
   unsigned bad = 0;
 
   __device__ __forceinline__ void add(const float (&o)[Q]) {
@@ -148,20 +184,27 @@ struct NodeTotals {
       if (ex(i)) df_add(jx, ex(i) > 0 ? o[i] : -o[i]);
       if (ey(i)) df_add(jy, ey(i) > 0 ? o[i] : -o[i]);
     }
-    df_norm(r);
-    df_norm(jx);
-    df_norm(jy);
-    const float en = 0.5f * (jx.hi * jx.hi + jy.hi * jy.hi) / r.hi;
-    df_add(m, r);
-    df_add(px, jx);
-    df_add(py, jy);
-    df_add(e, DF{en, 0.f});
+    if constexpr (Sum::kPair) {  // (three words take the node's two as they are)
+      df_norm(r);
+      df_norm(jx);
+      df_norm(jy);
+    }
+    // (the roundings spelled out: the same in every kernel that takes totals)
+    const float rh = __fadd_rn(r.hi, r.lo), jxh = __fadd_rn(jx.hi, jx.lo),
+                jyh = __fadd_rn(jy.hi, jy.lo);
+    const float en =
+        __fdiv_rn(__fmul_rn(0.5f, __fmaf_rn(jxh, jxh, __fmul_rn(jyh, jyh))), rh);
+    df_add(sm, r);
+    df_add(spx, jx);
+    df_add(spy, jy);
+    if constexpr (Sum::kPair) df_add(se, DF{en, 0.f}); else se.add(en);
   }
 
   // Sum over the block (NT threads) added to totals[0..4] in FP64.
   template <int NT>
   __device__ __forceinline__ void flush(double* __restrict__ totals) {
     __shared__ double red[NT / 32][5];
+    DF m = as_pair(sm), px = as_pair(spx), py = as_pair(spy), e = as_pair(se);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       df_add(m, df_shfl_xor(m, o));

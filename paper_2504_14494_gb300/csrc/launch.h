@@ -7,7 +7,7 @@
 namespace lbmgnn {
 
 // Launch that, with `early`, may start before the preceding kernel on `st` has
-// completed; the kernel waits for it in dep_sync() (common.cuh).  Early only
+// completed; the kernel waits for it in dep_wait() (common.cuh).  Early only
 // while the kernels of a call need one CTA per SM: the shared-memory split of
 // an SM cannot change under a running CTA, so the CTAs of a kernel that wants
 // two per SM, started early, ran one per SM (1024^2 GNN-LBM step 599 us
@@ -27,6 +27,9 @@ inline cudaError_t launch_after(bool early, void (*kern)(Params...), unsigned gr
   cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
 }
+
+// SMs of the current device; 0: unknown.
+int sm_count();
 
 cudaError_t launch_bgk_step(const float* fin, float* fout, const Shape& s, float tau,
                             const float* taus, double* totals, cudaStream_t st);

@@ -615,6 +615,8 @@ cudaError_t temporal(const float* src, float* dst, const Shape& s, float tau, co
   return vec ? temporal_t<T, 1, true>(a, st) : temporal_t<T, 1, false>(a, st);
 }
 
+}  // namespace
+
 int sm_count() {
   static std::atomic<int> cached[64];
   int dev = 0, n = 0;
@@ -626,8 +628,6 @@ int sm_count() {
   }
   return n;
 }
-
-}  // namespace
 
 cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const Shape& s, float tau,
                              const float* taus, int nsteps, cudaStream_t st) {
