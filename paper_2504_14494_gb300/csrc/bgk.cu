@@ -162,11 +162,13 @@ __global__ void __launch_bounds__(256) bgk_step_any(const float* __restrict__ fi
 }
 
 // ---------------------------------------------------------------------------
-// Moments of a stored state and FP64 totals.  A thread takes several nodes, 64
-// at most (the bound of a thread's sums, common.cuh): a block per 256 nodes
-// ended in 5 atomics on the same 5 words each, which bound the kernel (totals
-// of 1.6 M nodes: 49 us, now 25; of 4096^2: 441, now 173; 166 with two words
-// per sum).
+// Moments of a stored state and (TOTALS) its FP64 totals.  With totals a thread
+// takes several nodes, 64 at most (the bound of a thread's sums, common.cuh): a
+// block per 256 nodes ended in 5 atomics on the same 5 words each, which bound
+// the kernel (totals of 1.6 M nodes: 49 us, now 25; of 4096^2: 441, now 173; 166
+// with two words per sum).  The fields alone are bound by memory, and many
+// short blocks, a node per thread, do better there (4096^2: 115 us against 139).
+template <bool TOTALS>
 __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ f, Shape s,
                                                       float* __restrict__ rho,
                                                       float* __restrict__ ux,
@@ -175,8 +177,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ 
   dep_sync();
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   NodeTotals<TF> t;
-  for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N;
-       n += (int64_t)gridDim.x * blockDim.x) {
+  auto node = [&](int64_t n) {
     float v[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) v[q] = __ldg(f + q * s.ps + n);
@@ -184,11 +185,15 @@ __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ 
     if (rho) rho[n] = m.rho;
     if (ux) ux[n] = m.ux;
     if (uy) uy[n] = m.uy;
-    if (totals) t.add(v);
-  }
-  if (totals) {
+    if constexpr (TOTALS) t.add(v);
+  };
+  int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if constexpr (TOTALS) {
+    for (; n < N; n += (int64_t)gridDim.x * blockDim.x) node(n);
     if (t.bad) raise_status(stw, ST_NONFINITE);
     t.flush<256>(totals);
+  } else if (n < N) {
+    node(n);
   }
 }
 
@@ -260,10 +265,15 @@ cudaError_t launch_moments(const float* f, const Shape& s, float* rho, float* ux
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   unsigned* stw = status_word();
   if (totals && !stw) return cudaErrorInvalidDevice;
+  const int64_t per_node = (N + 255) / 256;
+  if (!totals) {
+    moments_kernel<false><<<(unsigned)per_node, 256, 0, st>>>(f, s, rho, ux, uy, nullptr, stw);
+    return cudaGetLastError();
+  }
   // 8 blocks per SM, more where a thread would take more than 64 nodes
   const int64_t few = std::max<int64_t>(8 * std::max(1, sm_count()), (N + 64 * 256 - 1) / (64 * 256));
-  const unsigned blocks = (unsigned)std::min<int64_t>((N + 255) / 256, few);
-  moments_kernel<<<blocks, 256, 0, st>>>(f, s, rho, ux, uy, totals, stw);
+  const unsigned blocks = (unsigned)std::min(per_node, few);
+  moments_kernel<true><<<blocks, 256, 0, st>>>(f, s, rho, ux, uy, totals, stw);
   return cudaGetLastError();
 }
 

@@ -82,3 +82,20 @@ def test_sum_over_the_nodes_of_one_thread(lbmlib, cuda, draw):
     want = count * (Fraction(hi.item()) + Fraction(lo.item()))
     err = abs(Fraction(t[0].item()) - want) / want
     assert err <= Fraction(11, 10) / 2 ** 48, float(err * 2 ** 48)
+
+
+@pytest.mark.parametrize("nx,ny,nb", [(1, 1, 1), (255, 1, 1), (257, 3, 2), (1023, 517, 3)])
+def test_fields_with_and_without_totals(lbmlib, cuda, nx, ny, nb):
+    """The two instances of the moments kernel give the same fields."""
+    import torch
+    L = lbmlib
+    n = nx * ny * nb
+    s = L.shape(nx, ny, nb)
+    f = _state(n, cuda, seed=nx)
+    got = [torch.full((n,), -7.0, device=cuda) for _ in range(6)]
+    L.lbm_moments(f, s, *got[:3])
+    L.lbm_moments(f, s, *got[3:], totals=torch.zeros(5, dtype=torch.float64, device=cuda))
+    for a, b in zip(got[:3], got[3:]):
+        assert torch.equal(a, b)
+    rho = f.view(9, n).double().sum(0)
+    assert float(((got[0].double() - rho).abs() / rho).max()) <= 8 * 2 ** -24
