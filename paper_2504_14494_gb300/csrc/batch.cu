@@ -14,7 +14,7 @@
 #include <string>
 #include <vector>
 
-#include "common.cuh"
+#include "collide.cuh"
 #include "gnn.cuh"
 #include "gnn_launch.h"
 #include "launch.h"

@@ -13,7 +13,7 @@
 #include <algorithm>
 #include <atomic>
 
-#include "common.cuh"
+#include "collide.cuh"
 #include "launch.h"
 
 namespace lbmgnn {

@@ -1,8 +1,9 @@
 // Several plain steps per launch: the multi-step calls of the BGK step (Eq. 1,
 // Eq. 2, Fig. 1 loop) and of the channel step, with the state kept on chip
-// between the steps.  Every node of every step is computed by the same
-// bgk_collide / channel_relax on the same nine pulled values as in the
-// single-step kernels, so the results are the same bit for bit.
+// between the steps.  Every node of every step is computed by the same BGK
+// formula with the same roundings (collide.cuh), or by the same channel_relax, on
+// the same nine pulled values as in the single-step kernels, so the results are
+// the same bit for bit.
 //
 // Two forms, chosen by estimated time (launch_bgk_steps):
 //
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, un
       float f[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) f[q] = sm[cur + src[k][q]];
-      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide_one(f, omega);
+      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide_fast(f, omega);
       if (last) {
         float* o = a.fout + lat + (int64_t)(ya - 1) * nx + own[k];
 #pragma unroll
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(32 * (T / S) * temporal_units<T / S>(),
   // hand-over slots and the p row to replace.
   auto iteration = [&](int i, auto par) {
     constexpr int PAR = decltype(par)::value;
-    float2 f[Q][1];
+    float2 f[Q];
     if (w == 0) {
       asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
       __syncwarp();  // every lane's copies of row i have landed
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(32 * (T / S) * temporal_units<T / S>(),
     {
       const float* r = w == 0 ? sm + (i % RING) * ROWF + 2 * lane : in_slot + (1 - PAR) * ROWF;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) f[q][0] = *reinterpret_cast<const float2*>(r + q * COLS);
+      for (int q = 0; q < Q; ++q) f[q] = *reinterpret_cast<const float2*>(r + q * COLS);
     }
     if (w == 0) fetch(i + AHEAD);  // into the slot of row i - 1, which every lane has read
 #pragma unroll
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(32 * (T / S) * temporal_units<T / S>(),
       float2 g[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        g[q] = f[q][0];
+        g[q] = f[q];
         if (ex(q) > 0)
           g[q] = make_float2(__shfl_up_sync(0xffffffffu, g[q].y, 1), g[q].x);
         else if (ex(q) < 0)
@@ -435,29 +436,29 @@ __global__ void __launch_bounds__(32 * (T / S) * temporal_units<T / S>(),
       }
       // e_y = -1 from the row just received, e_y = 0 from the one before it,
       // e_y = +1 from the one before that
-      f[0][0] = z[s][0], f[1][0] = z[s][1], f[3][0] = z[s][2];
-      f[2][0] = p[s][PAR][0], f[5][0] = p[s][PAR][1], f[6][0] = p[s][PAR][2];
-      f[4][0] = g[4], f[7][0] = g[7], f[8][0] = g[8];
+      f[0] = z[s][0], f[1] = z[s][1], f[3] = z[s][2];
+      f[2] = p[s][PAR][0], f[5] = p[s][PAR][1], f[6] = p[s][PAR][2];
+      f[4] = g[4], f[7] = g[7], f[8] = g[8];
       z[s][0] = g[0], z[s][1] = g[1], z[s][2] = g[3];
       p[s][PAR][0] = g[2], p[s][PAR][1] = g[5], p[s][PAR][2] = g[6];
-      bgk_collide_pairs(f, nomega);
+      bgk_collide_pair(f, nomega);
     }
     if (w < G - 1) {
       float* o = out_slot + PAR * ROWF;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * COLS) = f[q][0];
+      for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * COLS) = f[q];
     } else if (i >= 2 * T + G - 1) {  // lattice row y0 + i - (2 T + G - 1)
       float* o = out + (int64_t)(i - (2 * T + G - 1)) * nx;
       if constexpr (VEC) {
         if (vstore) {
 #pragma unroll
-          for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * ps + 2 * lane) = f[q][0];
+          for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(o + q * ps + 2 * lane) = f[q];
         }
       } else {
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < Q; ++q)
-          *reinterpret_cast<float2*>(stage_out + q * COLS + 2 * lane) = f[q][0];
+          *reinterpret_cast<float2*>(stage_out + q * COLS + 2 * lane) = f[q];
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 2; ++j) {

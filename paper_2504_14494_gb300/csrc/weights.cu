@@ -13,7 +13,7 @@
 //
 // Three deterministic passes: per (lattice, chunk) partial sums in FP64, one
 // fixed-order sum per lattice, and the mean and weights in one CTA.
-#include "common.cuh"
+#include "collide.cuh"
 #include "gnn.cuh"
 #include "gnn_launch.h"
 

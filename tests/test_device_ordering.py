@@ -122,3 +122,18 @@ def test_waits_for_another_cta_acquire_at_cluster_scope():
     assert senders == 1  # the resident multi-step kernel
     body = functions()["mbar_try_wait_sleep"][1]
     assert "try_wait.parity.acquire.cluster." in body[:body.index("else")]
+
+
+def test_collisions_spell_out_their_roundings():
+    """A product and a sum written with operators may or may not be contracted,
+    kernel by kernel; the BGK collision, which single-step and multi-step calls
+    share (equal bit for bit), uses none."""
+    funcs = functions()
+    for name in ("rho9", "mom9", "usq9", "feq_poly", "bgk_relax", "bgk_collide", "bgk_collide_fast",
+                 "bgk_collide_pair"):
+        body = funcs[name][1].replace("3.0f * sign", "")  # (exact: sign is +-1)
+        assert not re.search(r"[\w)\]] [*+-] [\w(]|[*+-]=", body), name
+    src = "".join(_strip(open(p).read()) for p in glob.glob(os.path.join(CSRC, "*.cu*")))
+    assert len(re.findall(r"void bgk_collide\(", src)) == 1
+    for kernel in ("bgk_step_x4", "bgk_step_any", "bgk_batch_kernel", "pair_residual_kernel"):
+        assert "bgk_collide(" in funcs[kernel][1], kernel
