@@ -86,6 +86,13 @@ LBM_API int lbm_get_status(void* stream);
  * LBM_ERR_TIMEOUT.  Nothing traps or hangs. */
 LBM_API int lbm_selftest_wait_timeout(long long max_cycles, void* stream);
 
+/* Self-test of the reciprocals that the collisions use in place of a division
+ * (no counterpart in the paper): every float against the IEEE quotient 1/x.
+ *   bad  device, two counts, overwritten: floats for which the packed
+ *        reciprocal (|x| in [2^-100, 2^100]) and the scalar one (any x) differ
+ *        from it; both are 0. */
+LBM_API int lbm_selftest_reciprocal(unsigned long long* bad, void* stream);
+
 /* Taylor-Green vortex initial state (paper Sec. 3.2; the formula is this
  * library's reading): u_x = u0 cos(kx x) sin(ky y), u_y = -u0 sin(kx x)
  * cos(ky y) at integer node coordinates, rho = rho0 or, if

@@ -54,6 +54,7 @@ _SIGS = {
     "lbm_version": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "lbm_get_status": (ctypes.c_int, [_VP]),
     "lbm_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_longlong, _VP]),
+    "lbm_selftest_reciprocal": (ctypes.c_int, [_VP, _VP]),
     "lbm_init_tgv": (ctypes.c_int, [_VP, lbm_shape, ctypes.c_double, ctypes.c_double,
                                     ctypes.c_double, ctypes.c_double, ctypes.c_int, _VP]),
     "lbm_step_bgk": (ctypes.c_int, [_VP, _VP, _VP, lbm_shape, ctypes.c_float, _VP, ctypes.c_int,
@@ -271,6 +272,11 @@ def lbm_get_status(stream=None):
 def lbm_selftest_wait_timeout(max_cycles, stream=None):
     check(load().lbm_selftest_wait_timeout(int(max_cycles), stream_ptr(stream)),
           "lbm_selftest_wait_timeout")
+
+
+def lbm_selftest_reciprocal(bad, stream=None):
+    check(load().lbm_selftest_reciprocal(dptr(bad, "bad", _torch().int64, 2), stream_ptr(stream)),
+          "lbm_selftest_reciprocal")
 
 
 def lbm_init_tgv(f, s, rho0, u0, kx, ky, pressure_consistent=False, stream=None):
