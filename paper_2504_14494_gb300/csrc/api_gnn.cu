@@ -262,7 +262,7 @@ int gnn_forward(const float* f_pre, lbm_shape shape, const void* packed, void* s
   __nv_bfloat16* a1 = a0 + N * 64;
   __half* ab0 = reinterpret_cast<__half*>(a1 + N * 64);
   __half* ab1 = ab0 + N * 128;
-  if (launch_gnn_encode(f_pre, false, false, s, pk, h0, ab0, st) != cudaSuccess)
+  if (launch_gnn_encode(f_pre, s, pk, h0, ab0, st) != cudaSuccess)
     return LBM_ERR_CUDA;
   RoundLaunch r0;
   r0.h_in = h0;

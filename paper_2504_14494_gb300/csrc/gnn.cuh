@@ -51,7 +51,7 @@ constexpr uint32_t NORM = 3584;   // fp32 mu[12], sigma[12], s_df, variant, pad,
 constexpr uint32_t BH = 3712;     // fp32 [16] (10 used)
 constexpr uint32_t WHF = 3776;    // fp32 [10][64] (BF16-rounded values)
 constexpr uint32_t W2 = 7168;     // SW128 [64 out x 64 in]
-constexpr uint32_t W2T = 15360;   // SW128 [64 in x 64 out]
+constexpr uint32_t W2T = 15360;   // SW128 [64 in x 64 out] (layout version 1 holds it; no kernel reads it)
 constexpr uint32_t WH = 23552;    // SW128 [16 out (10 used) x 64 in]
 constexpr uint32_t ROUND0 = 25600;
 constexpr uint32_t ROUND_SIZE = 68608;
@@ -59,7 +59,7 @@ constexpr uint32_t ROUND_SIZE = 68608;
 constexpr uint32_t WAB = 0;        // SW128 [128 out (a rows, then b rows) x 64 in]
 constexpr uint32_t WABT = 16384;   // 2 SW128 blocks [64 in x 64 out], block kb = W_a / W_b
 constexpr uint32_t WN = 32768;     // 2 SW128 blocks [64 out x 64 in], block 0: h part, 1: a part
-constexpr uint32_t WNT = 49152;    // SW128 [128 in x 64 out]
+constexpr uint32_t WNT = 49152;    // SW128 [128 in x 64 out] (as W2T: read by no kernel)
 constexpr uint32_t CK = 65536;     // fp32 [8][64]: c_k = W_c e_k + b_e, k = 1..8
 constexpr uint32_t BE = 67584;     // fp32 [64]
 constexpr uint32_t BN = 67840;     // fp32 [64]
@@ -357,12 +357,7 @@ __device__ __forceinline__ const float4* chunk4(const float* base, int64_t N, in
 __device__ __forceinline__ float4* chunk4w(float* base, int64_t N, int64_t n, int f) {
   return reinterpret_cast<float4*>(base + ((int64_t)(f >> 2) * N + n) * 4);
 }
-// 32 BF16 values (features f0..f0+31) of node n / their store.
-__device__ __forceinline__ void ld_pb32(const __nv_bfloat16* base, int64_t N, int64_t n, int f0,
-                                        float* v) {
-#pragma unroll
-  for (int c = 0; c < 4; ++c) unpack_bf16x8(ld_prev(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
-}
+// Store of 32 BF16 values (features f0..f0+31) of node n.
 __device__ __forceinline__ void st_pb32(__nv_bfloat16* base, int64_t N, int64_t n, int f0,
                                         const float* v) {
 #pragma unroll
@@ -407,12 +402,6 @@ __device__ __forceinline__ void st_pf(float* base, int64_t N, int64_t n, int f0,
 #pragma unroll
   for (int c = 0; c < NF / 4; ++c)
     *chunk4w(base, N, n, f0 + 4 * c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-}
-template <int NF>
-__device__ __forceinline__ void ld_pb(const __nv_bfloat16* base, int64_t N, int64_t n, int f0,
-                                      float* v) {
-#pragma unroll
-  for (int c = 0; c < NF / 8; ++c) unpack_bf16x8(ld_prev(chunk8(base, N, n, f0 + 8 * c)), v + 8 * c);
 }
 template <int NF>
 __device__ __forceinline__ void st_pb(__nv_bfloat16* base, int64_t N, int64_t n, int f0,

@@ -141,16 +141,9 @@ constexpr uint32_t W1X = 0, W2 = 8192, WAB = 16384, X1 = 32768, X = 49152, B1 = 
 #ifndef LBM_ENC_CTAS
 #define LBM_ENC_CTAS 2  // resident encoder CTAs per SM
 #endif
-// The inference encoder (pull, B only) runs 3 CTAs per SM at 80 registers:
-// for one stack of lattices without spilling (the step 2 % faster), for the
-// table geometry of batched runs with a few spilled values and still 3 %
-// faster; the training instances would spill more and keep LBM_ENC_CTAS.
-template <bool PULL, bool BONLY, class Geo>
-constexpr int enc_ctas() {
-  return (PULL && BONLY) ? 3 : LBM_ENC_CTAS;
-}
-template <bool PULL, bool BONLY, class Geo>
-__global__ void __launch_bounds__(256, (enc_ctas<PULL, BONLY, Geo>())) gnn_encode_kernel(
+// (The training forward's encoder; an inference step has that of gnn_mlp.cu.)
+template <class Geo>
+__global__ void __launch_bounds__(256, LBM_ENC_CTAS) gnn_encode_kernel(
     const float* __restrict__ f, Geo geo, const uint8_t* __restrict__ packed,
     __nv_bfloat16* __restrict__ h0_out, __half* __restrict__ ab_out, unsigned* stw) {
   if (!blob_ok(packed, stw)) return dep_sync();
@@ -180,19 +173,12 @@ __global__ void __launch_bounds__(256, (enc_ctas<PULL, BONLY, Geo>())) gnn_encod
   const int64_t ntiles = (N + TILE - 1) / TILE;
   const bool relu = variant_of(nrm) & VAR_MLP_ONLY;
 
-  // populations of node `t * TILE + node` of tile t (streamed when PULL)
+  // populations of node `t * TILE + node` of tile t
   auto load_f = [&](int64_t t, float (&v)[Q]) {
     const int64_t m = t * TILE + node;
     const int64_t mm = m < N ? m : N - 1;
-    if (PULL) {
-      const GeoPos p = geo.pos(base + mm);
 #pragma unroll
-      for (int q = 0; q < Q; ++q)
-        v[q] = __ldg(f + q * ps + checked(geo_nbr(p, -ex(q), -ey(q)), base, base + N, stw));
-    } else {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) v[q] = __ldg(f + q * ps + base + mm);
-    }
+    for (int q = 0; q < Q; ++q) v[q] = __ldg(f + q * ps + base + mm);
   };
   float fnext[Q];
   dep_sync();
@@ -248,22 +234,15 @@ __global__ void __launch_bounds__(256, (enc_ctas<PULL, BONLY, Geo>())) gnn_encod
     bias_act(g, b2 + f0, 32, relu);
     if (on && h0_out) st_pb32(h0_out, N, n, f0, g);
     st_row32(X, node, f0, g);  // the MMA that read X has completed
-    // A | B = h0 [W_a; W_b]^T ([N][128]), or B alone ([N][64]) when BONLY
-    // (inference; nothing at all for the MLP-only network, which passes no
-    // messages)
-    if (!(BONLY && relu)) {
-      if (!tc_run(sh, tc, stw, [&] {
-            umma_128xN(tc.tmem, smem_u32(X), 0, smem_u32(sm + enc::WAB) + (BONLY ? 8192 : 0), 0, 1,
-                       BONLY ? 64 : 128, false);
-          }))
-        break;
-      tmem_ld32(lb + f0, g);
-      if (on) st_ph32(ab_out, N, n, f0, g);
-      if (!BONLY) {
-        tmem_ld32(lb + HID + f0, g);
-        if (on) st_ph32(ab_out, N, n, HID + f0, g);
-      }
-    }
+    // A | B = h0 [W_a; W_b]^T ([N][128])
+    if (!tc_run(sh, tc, stw, [&] {
+          umma_128xN(tc.tmem, smem_u32(X), 0, smem_u32(sm + enc::WAB), 0, 1, 128, false);
+        }))
+      break;
+    tmem_ld32(lb + f0, g);
+    if (on) st_ph32(ab_out, N, n, f0, g);
+    tmem_ld32(lb + HID + f0, g);
+    if (on) st_ph32(ab_out, N, n, HID + f0, g);
 #if !LBM_PREFETCH
     if (tile + gridDim.x < ntiles) load_f(tile + gridDim.x, fnext);
 #endif
@@ -608,30 +587,16 @@ cudaError_t launch_gnn_pack(const float* params, uint8_t* packed, cudaStream_t s
 }
 
 
-template <bool PULL, bool BONLY, class Geo>
-static cudaError_t encode_t(const float* f, const Geo& geo, int64_t N, int per_sm,
-                           uint32_t bytes, const uint8_t* packed, __nv_bfloat16* h0, __half* ab,
-                           unsigned* stw, cudaStream_t st) {
-  const unsigned grid = grid_for(N, per_sm >= 2 ? enc_ctas<PULL, BONLY, Geo>() : per_sm);
-  cudaError_t e;
-  if ((e = set_smem(gnn_encode_kernel<PULL, BONLY, Geo>, bytes)) != cudaSuccess) return e;
-  gnn_encode_kernel<PULL, BONLY, Geo><<<grid, 256, bytes, st>>>(f, geo, packed, h0, ab, stw);
-  return cudaGetLastError();
-}
-
-// pull: f is a stored state (stream first); b_only: write B alone ([N][64]).
 template <class Geo>
-static cudaError_t encode_any(const float* f, bool pull, bool b_only, const Geo& geo, int64_t N,
-                              const uint8_t* packed, __nv_bfloat16* h0, __half* ab,
-                              cudaStream_t st, int per_sm = 2) {
+static cudaError_t encode_t(const float* f, const Geo& geo, int64_t N, const uint8_t* packed,
+                            __nv_bfloat16* h0, __half* ab, cudaStream_t st) {
   unsigned* stw = status_word();
   if (!stw) return cudaErrorInvalidDevice;
   const uint32_t bytes = enc::BYTES + 1024;
-  if (pull)
-    return b_only ? encode_t<true, true>(f, geo, N, per_sm, bytes, packed, h0, ab, stw, st)
-                  : encode_t<true, false>(f, geo, N, per_sm, bytes, packed, h0, ab, stw, st);
-  return b_only ? encode_t<false, true>(f, geo, N, per_sm, bytes, packed, h0, ab, stw, st)
-                : encode_t<false, false>(f, geo, N, per_sm, bytes, packed, h0, ab, stw, st);
+  cudaError_t e;
+  if ((e = set_smem(gnn_encode_kernel<Geo>, bytes)) != cudaSuccess) return e;
+  gnn_encode_kernel<Geo><<<grid_for(N, LBM_ENC_CTAS), 256, bytes, st>>>(f, geo, packed, h0, ab, stw);
+  return cudaGetLastError();
 }
 
 template <int MODE, int T, int G, bool AH, class Geo>
@@ -684,11 +649,9 @@ static cudaError_t round_step(int mode, const RoundLaunch& rl, const Geo& geo, i
                    : round_t<1, true>(round_args(rl), geo, N, per_sm, packed, stw, st);
 }
 
-cudaError_t launch_gnn_encode(const float* f, bool pull, bool b_only, const Shape& s,
-                              const uint8_t* packed, __nv_bfloat16* h0, __half* ab,
-                              cudaStream_t st) {
-  return encode_any(f, pull, b_only, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx, packed, h0, ab,
-                    st);
+cudaError_t launch_gnn_encode(const float* f, const Shape& s, const uint8_t* packed,
+                              __nv_bfloat16* h0, __half* ab, cudaStream_t st) {
+  return encode_t(f, make_geo_stack(s), (int64_t)s.nb * s.ny * s.nx, packed, h0, ab, st);
 }
 
 cudaError_t launch_gnn_round(int mode, const RoundLaunch& rl, const Shape& s,
@@ -718,9 +681,7 @@ cudaError_t launch_gnn_forward_channel(const float* f_pre, const Shape& s, float
   geo.fxs = forces_x;
   const int64_t N = (int64_t)s.nb * s.ny * s.nx;
   cudaError_t e;
-  if ((e = encode_t<false, false>(f_pre, geo, N, 2, enc::BYTES + 1024, packed, sv.h0, sv.ab0, stw,
-                                  st)) != cudaSuccess)
-    return e;
+  if ((e = encode_t(f_pre, geo, N, packed, sv.h0, sv.ab0, st)) != cudaSuccess) return e;
   RoundArgs r0{sv.h0, sv.ab0, sv.h1, sv.a0, sv.ab1, nullptr, nullptr, nullptr, 1.0f, nullptr, 0,
                nullptr};
   if ((e = round_t<0, false>(r0, geo, N, 2, packed, stw, st)) != cudaSuccess) return e;

@@ -27,10 +27,9 @@ struct RoundLaunch {
 };
 
 cudaError_t launch_gnn_pack(const float* params, uint8_t* packed, cudaStream_t st);
-// pull: f is a stored state (streamed first); b_only: ab receives B alone.
-cudaError_t launch_gnn_encode(const float* f, bool pull, bool b_only, const Shape& s,
-                              const uint8_t* packed, __nv_bfloat16* h0, __half* ab,
-                              cudaStream_t st);
+// The training forward's encoder: h0 and A | B of pre-collision populations f.
+cudaError_t launch_gnn_encode(const float* f, const Shape& s, const uint8_t* packed,
+                              __nv_bfloat16* h0, __half* ab, cudaStream_t st);
 // mode 0: inner round; 1: last round + head + Eq. 3 collision; 2: last round + head -> y
 cudaError_t launch_gnn_round(int mode, const RoundLaunch& rl, const Shape& s,
                              const uint8_t* packed, cudaStream_t st);

@@ -276,7 +276,8 @@ cudaError_t resident(const ResidentArgs& a, const ResidentPlan& p, cudaStream_t 
     switch (p.kn) {
       case 1: return resident_t<CH, 1, true>(a, p, st);
       case 2: return resident_t<CH, 2, true>(a, p, st);
-      default: return resident_t<CH, 3, true>(a, p, st);
+      // (one CTA takes at most 512 nodes, or one row, of which 1,075 nodes fit)
+      default: return cudaErrorInvalidConfiguration;
     }
   }
   switch (p.kn) {
