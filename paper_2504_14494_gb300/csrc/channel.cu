@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) channel_step_kernel(const float* __restri
   const NodeIdx i = node_idx(s);
   float f[Q];
   channel_pull(fin, s, i.nn, i.x, i.y, i.lat, f, stw);
-  channel_relax(f, taus ? __ldg(taus + i.b) : tau, gx);
+  channel_relax<false>(f, taus ? __ldg(taus + i.b) : tau, gx);
   if (i.on) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) fout[q * s.ps + i.nn] = f[q];
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(256) channel_gnn_collide_kernel(
   for (int q = 0; q < Q; ++q) d[q] = sdf * __ldg(y + (int64_t)(1 + q) * N + i.nn);
   if (variant & VAR_CONSERVATIVE) conserve9(d);
   const float t = (taus ? __ldg(taus + i.b) : tau) * tau_adj_of(__ldg(y + i.nn), variant);
-  channel_relax(f, t, gx);
+  channel_relax<false>(f, t, gx);
 #pragma unroll
   for (int q = 0; q < Q; ++q) f[q] += d[q];
   if (i.on) {

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(1024) resident_steps_kernel(ResidentArgs a, un
       float f[Q];
 #pragma unroll
       for (int q = 0; q < Q; ++q) f[q] = sm[cur + src[k][q]];
-      if constexpr (CH) channel_relax(f, tau, a.gx); else bgk_collide_fast(f, omega);
+      if constexpr (CH) channel_relax<true>(f, tau, a.gx); else bgk_collide_fast(f, omega);
       if (last) {
         float* o = a.fout + lat + (int64_t)(ya - 1) * nx + own[k];
 #pragma unroll
