@@ -169,10 +169,7 @@ int lbm_step_bgk(const float* f_in, float* f_out, float* f_tmp, lbm_shape shape,
   }
   if (nsteps == 1)
     return cuda_status(launch_bgk_step(f_in, f_out, s, tau, taus, totals, st));
-  if (launch_bgk_steps(f_in, f_out, f_tmp, s, tau, taus, nsteps, st) != cudaSuccess)
-    return LBM_ERR_CUDA;
-  return totals ? cuda_status(launch_moments(f_out, s, nullptr, nullptr, nullptr, totals, st))
-                : LBM_OK;
+  return cuda_status(launch_bgk_steps(f_in, f_out, f_tmp, s, tau, taus, nsteps, totals, st));
 }
 
 int lbm_step_channel(const float* f_in, float* f_out, float* f_tmp, lbm_shape shape, float tau,
@@ -201,9 +198,10 @@ int lbm_step_channel(const float* f_in, float* f_out, float* f_tmp, lbm_shape sh
   }
   const float* src = f_in;
   int done = 0;
-  if (nsteps > 1 && channel_steps_fit(s, nsteps)) {
-    // all steps on chip, but for a last one with totals (by the single-step kernel)
-    done = totals ? nsteps - 1 : nsteps;
+  // all steps on chip, but for a last one with totals (by the single-step kernel)
+  const int chip = totals ? nsteps - 1 : nsteps;
+  if (nsteps > 1 && channel_steps_fit(s, chip, st)) {
+    done = chip;
     float* dst = totals ? f_tmp : f_out;
     if (launch_channel_steps(f_in, dst, s, tau, taus, force_x, done, st) != cudaSuccess)
       return LBM_ERR_CUDA;

@@ -228,6 +228,15 @@ static inline bool x4_ok(const float* a, const float* b, const Shape& s) {
          ((uintptr_t)b % 16 == 0);
 }
 
+// Blocks of a step of `rows` rows: 4 warps of up to 128 nodes of a row, or 256 nodes.
+static int64_t step_blocks(bool x4, const Shape& s, int64_t rows) {
+  return x4 ? (rows * ((s.nx + 127) / 128) + 3) / 4 : (rows * s.nx + 255) / 256;
+}
+
+int64_t bgk_step_blocks(const float* fin, const float* fout, const Shape& s) {
+  return step_blocks(x4_ok(fin, fout, s), s, (int64_t)s.nb * s.ny);
+}
+
 cudaError_t launch_bgk_step_rows(const float* fin, float* fout, const Shape& s, float tau,
                                  const float* taus, double* totals, int64_t row0, int64_t row1,
                                  cudaStream_t st) {
@@ -235,16 +244,15 @@ cudaError_t launch_bgk_step_rows(const float* fin, float* fout, const Shape& s, 
   unsigned* stw = status_word();
   if (totals && !stw) return cudaErrorInvalidDevice;
   const int64_t rows = row1 - row0;
-  if (x4_ok(fin, fout, s)) {
-    const int64_t warps = rows * ((s.nx + 127) / 128);
-    const unsigned blocks = (unsigned)((warps + 3) / 4);
+  const bool x4 = x4_ok(fin, fout, s);
+  const unsigned blocks = (unsigned)step_blocks(x4, s, rows);
+  if (x4) {
     if (totals)
       bgk_step_x4<true><<<blocks, 128, 0, st>>>(fin, fout, s, tau, taus, totals, stw, row0, row1);
     else
       bgk_step_x4<false><<<blocks, 128, 0, st>>>(fin, fout, s, tau, taus, totals, stw, row0,
                                                  row1);
   } else {
-    const unsigned blocks = (unsigned)((rows * s.nx + 255) / 256);
     if (totals)
       bgk_step_any<true><<<blocks, 256, 0, st>>>(fin, fout, s, tau, taus, totals, stw, row0,
                                                  row1);

@@ -31,6 +31,8 @@ inline cudaError_t launch_after(bool early, void (*kern)(Params...), unsigned gr
 // SMs of the current device; 0: unknown.
 int sm_count();
 
+// Blocks of a single step of these buffers (each ends in 5 atomics with totals).
+int64_t bgk_step_blocks(const float* fin, const float* fout, const Shape& s);
 cudaError_t launch_bgk_step(const float* fin, float* fout, const Shape& s, float tau,
                             const float* taus, double* totals, cudaStream_t st);
 // The step restricted to lattice rows row0 .. row1-1 (of the nb*ny rows).
@@ -38,11 +40,12 @@ cudaError_t launch_bgk_step_rows(const float* fin, float* fout, const Shape& s, 
                                  const float* taus, double* totals, int64_t row0, int64_t row1,
                                  cudaStream_t st);
 // nsteps >= 2 BGK steps with the state kept on chip between steps
-// (multi_step.cu); ftmp: ping-pong buffer as in lbm_step_bgk.
+// (multi_step.cu); ftmp: ping-pong buffer as in lbm_step_bgk; totals of the last
+// state (cleared by the caller) or NULL.
 cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const Shape& s, float tau,
-                             const float* taus, int nsteps, cudaStream_t st);
+                             const float* taus, int nsteps, double* totals, cudaStream_t st);
 // The same for the channel step, for calls that channel_steps_fit() accepts.
-bool channel_steps_fit(const Shape& s, int nsteps);
+bool channel_steps_fit(const Shape& s, int nsteps, cudaStream_t st);
 cudaError_t launch_channel_steps(const float* fin, float* fout, const Shape& s, float tau,
                                  const float* taus, float gx, int nsteps, cudaStream_t st);
 cudaError_t launch_moments(const float* f, const Shape& s, float* rho, float* ux, float* uy,

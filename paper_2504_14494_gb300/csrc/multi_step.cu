@@ -491,13 +491,29 @@ cudaError_t temporal_t(TemporalArgs a, cudaStream_t st) {
 }
 
 // ---- which form -------------------------------------------------------------
-// Estimated times in microseconds, fitted to sweeps of 64^2 .. 4096^2 lattices
+// Estimated times in microseconds, fitted to sweeps of 32^2 .. 4096^2 lattices
 // and stacks on a GB300 (152 SMs): a step of the single-step kernel (4.1 per
 // launch; 7.3e-6 per node out of L2, 10.45e-6 out of HBM), a step of the
 // resident form, and a pass of the temporal form.  They only rank the forms.
-double single_us(const Shape& s) {
+//
+// Captured launches (`cap`) cost less than those the host makes one by one, a
+// single step of a small lattice 2.3 instead of 4.1, so that more calls are
+// best made of single steps: a 200^2 channel's 5 steps 14 us in a graph, 23 by
+// the resident form (eager: 21 and 25); 512^2 BGK, 10 steps, 38 and 39 (62 and
+// 45).
+bool is_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return c != cudaStreamCaptureStatusNone;
+}
+
+double single_us(const Shape& s, bool cap) {
   const double n = (double)s.nb * s.ny * s.nx;
-  return std::max({4.1, 3.0 + 7.3e-6 * n, 10.45e-6 * n});
+  return cap ? std::max({2.3, 1.9 + 7.0e-6 * n, 10.45e-6 * n})
+             : std::max({4.1, 3.0 + 7.3e-6 * n, 10.45e-6 * n});
 }
 
 // Clusters of 16 CTAs (more than every device takes) that run at once on this
@@ -538,14 +554,22 @@ int clusters16() {
 // (about 16 of 8 CTAs run at once, of 16 CTAs what the device says) 4 to load
 // and store; per step the chain of one node and the exchange, and the nodes of
 // a CTA (more than one per thread at half the rate; clusters of 16 fitted by
-// themselves: 64^2, 100 x 96, 128^2, 200^2).
-double resident_us(const Shape& s, const ResidentPlan& p, int nsteps) {
-  const int at_once = p.C == 16 ? std::max(1, clusters16()) : 128 / p.C;
+// themselves: 64^2, 100 x 96, 128^2, 200^2).  The channel's collision (`ch`)
+// takes 1.3 to 1.5 times as long per node: a step of 200^2 3.25 us against 2.6,
+// of 128^2 1.14 against 0.86, of 100^2 1.87 against 1.38; its stacks are counted
+// with the CTAs that share an SM (64 registers per thread).
+double resident_us(const Shape& s, const ResidentPlan& p, int nsteps, bool ch, bool cap) {
+  int at_once = p.C == 16 ? std::max(1, clusters16()) : 128 / p.C;
+  if (ch && p.C < 16)
+    at_once *= std::max(1, std::min(1024 / p.threads, (int)(SMEM_MAX / resident_smem(p.rows, s.nx))));
   const double waves = (double)((s.nb + at_once - 1) / at_once);
   const double nodes = (double)p.rows * s.nx;
-  const double step = p.C == 16 ? std::max(0.37, 0.24 + (p.kn == 1 ? 0.64e-3 : 0.91e-3) * nodes)
-                                : (p.C == 1 ? 0.20 : 0.38) + (p.kn == 1 ? 0.31e-3 : 0.73e-3) * nodes;
-  return 4.0 + waves * (4.0 + nsteps * step);
+  const double one = ch ? (p.C == 16 ? 0.88e-3 : 0.42e-3) : (p.C == 16 ? 0.64e-3 : 0.31e-3);
+  const double more = ch ? (p.C == 16 ? 1.16e-3 : 1.13e-3) : (p.C == 16 ? 0.91e-3 : 0.73e-3);
+  const double node = (p.kn == 1 ? one : more) * nodes;
+  const double step =
+      p.C == 16 ? std::max(0.37, 0.24 + node) : (p.C == 1 ? 0.20 : 0.38) + node;
+  return (cap ? 0.0 : 4.0) + waves * ((cap ? 3.3 : 4.0) + nsteps * step);
 }
 
 // The fastest by that estimate.  One CTA up to 512 nodes without an exchange
@@ -554,13 +578,15 @@ double resident_us(const Shape& s, const ResidentPlan& p, int nsteps) {
 // 128^2 1.09 against 2.08 (several steps per pass), four 100 x 96 1.05 against
 // 1.69; at 32^2 nothing is left to halve (0.38 against 0.36), and fewer run at
 // once (one per GPC), so that stacks stay with 8.
-ResidentPlan plan_resident(const Shape& s, int nsteps) {
+ResidentPlan plan_resident(const Shape& s, int nsteps, bool ch, bool cap) {
   const int64_t all = (int64_t)s.nx * s.ny;
   if (all > 16 * 3072) return {0, 0, 0, 0};
   ResidentPlan p = plan_resident_from(s, all <= 512 ? 1 : 8);
   if (all > 1024 && s.ny >= 16 && clusters16() > 0) {
     const ResidentPlan w = plan_resident_from(s, 16);
-    if (w.C == 16 && (!p.C || resident_us(s, w, nsteps) < resident_us(s, p, nsteps))) p = w;
+    if (w.C == 16 &&
+        (!p.C || resident_us(s, w, nsteps, ch, cap) < resident_us(s, p, nsteps, ch, cap)))
+      p = w;
   }
   return p;
 }
@@ -576,11 +602,16 @@ struct TemporalPlan {
 // warp: 0.33 alone, 0.89 at 24 warps; four stages in one warp: 0.65 alone,
 // 1.54 at 12), at least what HBM takes for the state once in and out.  The
 // range heights tried are those that give 1, 2, .. CTAs per SM and whole
-// waves: short ranges fill the SMs, long ones recompute fewer rows.
-TemporalPlan plan_temporal(const Shape& s, int T, int sms) {
+// waves: short ranges fill the SMs, long ones recompute fewer rows.  Captured: 2
+// less for the launch, but up to 2.5 more between 50 and 500 thousand nodes,
+// where an eager pass hides them behind its launch.
+TemporalPlan plan_temporal(const Shape& s, int T, int sms, bool cap) {
   TemporalPlan best;
   const int strips = (s.nx + COLS - 2 * HALO - 1) / (COLS - 2 * HALO);
   const int64_t cols = (int64_t)s.nb * strips;
+  const double nodes = (double)s.nb * s.ny * s.nx;
+  const double fixed =
+      cap ? 2.5 + std::min(2.5, 6e-6 * std::max(0.0, nodes - 5e4)) : 4.5;
   for (int form = 0; form < 2; ++form) {
     const bool one = form == 0;
     const int most = one ? 12 : 24 / T;           // strips' CTAs (warps) per SM
@@ -599,8 +630,7 @@ TemporalPlan plan_temporal(const Shape& s, int T, int sms) {
       const double it = one ? std::max(0.25 + 0.1 * T, 0.25 * T * (0.25 + 0.108 * warps))
                             : std::max(0.33, 0.22 + 0.0278 * warps);
       const double us =
-          std::max(4.5 + waves * it * (h + 2 * T + (one ? 0 : T - 1)),
-                   13.5e-6 * (double)s.nb * s.ny * s.nx);  // (HBM)
+          std::max(fixed + waves * it * (h + 2 * T + (one ? 0 : T - 1)), 13.5e-6 * nodes);  // (HBM)
       if (us < best.us) best = {us, one, strips, segs, h};
     }
   }
@@ -617,6 +647,79 @@ cudaError_t temporal(const float* src, float* dst, const Shape& s, float tau, co
   return vec ? temporal_t<T, 1, true>(a, st) : temporal_t<T, 1, false>(a, st);
 }
 
+// `nsteps` steps as one resident launch or as passes of 1 to MOST steps: the
+// fewest microseconds in all, for the last ones (up to TAIL) exactly, before
+// them passes of the cheapest kind per step.
+constexpr int MOST = 4, TAIL = 12;
+struct StepsPlan {
+  double us = 0.0;
+  ResidentPlan resident{0, 0, 0, 0};  // C = 0: by passes
+  TemporalPlan pass[MOST + 1];
+  int head = 0, head_steps = 1, tail = 0, passes = 0;  // head passes of head_steps, then `tail` steps
+  int first[TAIL + 1] = {0};                            // steps of the next pass with n left
+};
+StepsPlan plan_steps(const Shape& s, int nsteps, int sms, bool cap) {
+  StepsPlan p;
+  double us[MOST + 1] = {0.0, single_us(s, cap)};
+  const bool wide = s.nx >= (1 << 30) || s.ny >= (1 << 30);  // 32-bit rows and columns
+  for (int T = 2; T <= MOST && T <= nsteps; ++T) {
+    if (!wide) p.pass[T] = plan_temporal(s, T, sms, cap);
+    us[T] = p.pass[T].us;
+    if (us[T] / T < us[p.head_steps] / p.head_steps) p.head_steps = T;
+  }
+  p.tail = nsteps;
+  if (nsteps > TAIL) {
+    p.head = (nsteps - TAIL + p.head_steps - 1) / p.head_steps;
+    p.tail -= p.head * p.head_steps;
+  }
+  double cost[TAIL + 1] = {0.0};
+  for (int n = 1; n <= p.tail; ++n) {
+    cost[n] = 1e30;
+    for (int T = 1; T <= MOST && T <= n; ++T)
+      if (cost[n - T] + us[T] < cost[n]) cost[n] = cost[n - T] + us[T], p.first[n] = T;
+  }
+  p.us = p.head * us[p.head_steps] + cost[p.tail];
+  p.passes = p.head;
+  for (int n = p.tail; n > 0; n -= p.first[n]) ++p.passes;
+  if (nsteps > 1) {
+    const ResidentPlan rp = plan_resident(s, nsteps, false, cap);
+    const double rus = rp.C ? resident_us(s, rp, nsteps, false, cap) : 1e30;
+    if (rus < p.us) p.us = rus, p.resident = rp;
+  }
+  return p;
+}
+
+cudaError_t run_steps(const StepsPlan& p, const float* fin, float* fout, float* ftmp,
+                      const Shape& s, float tau, const float* taus, int nsteps, cudaStream_t st) {
+  if (p.resident.C) {
+    const ResidentArgs a{fin, fout, s, tau, taus, 0.0f, nsteps, p.resident.rows};
+    return resident<false>(a, p.resident, st);
+  }
+  // ping-pong so that the last pass lands in fout
+  const float* src = fin;
+  int left = p.tail;
+  for (int k = 0; k < p.passes; ++k) {
+    const int T = k < p.head ? p.head_steps : p.first[left];
+    if (k >= p.head) left -= T;
+    float* dst = (p.passes - k) % 2 == 1 ? fout : ftmp;
+    cudaError_t e = cudaSuccess;
+    switch (T) {
+      case 1: e = launch_bgk_step(src, dst, s, tau, taus, nullptr, st); break;
+      case 2: e = temporal<2>(src, dst, s, tau, taus, p.pass[2], st); break;
+      case 3: e = temporal<3>(src, dst, s, tau, taus, p.pass[3], st); break;
+      default: e = temporal<4>(src, dst, s, tau, taus, p.pass[4], st); break;
+    }
+    if (e != cudaSuccess) return e;
+    src = dst;
+  }
+  return cudaSuccess;
+}
+
+// What totals add: a pass of the moments kernel over the final state, or, to a
+// single step that takes them along, 5 atomics per block.
+double moments_us(double n) { return std::min(4.0 + 28e-6 * n, 9.0 + 10e-6 * n); }
+double fused_totals_us(double blocks) { return 2.8 + 5e-3 * blocks; }
+
 }  // namespace
 
 int sm_count() {
@@ -631,77 +734,46 @@ int sm_count() {
   return n;
 }
 
+// With totals the last step may be a single one that takes them along: better
+// for few steps of a small lattice (512^2, 2 steps: 17 us against 24 with a
+// pass for the totals after both), while a pass pays where it costs less than
+// the atomics of a single step and what that step would save inside a pass of
+// several (2048^2, 4096^2, 1.6 M odd nodes).
 cudaError_t launch_bgk_steps(const float* fin, float* fout, float* ftmp, const Shape& s, float tau,
-                             const float* taus, int nsteps, cudaStream_t st) {
-  constexpr int MOST = 4;  // steps per pass
+                             const float* taus, int nsteps, double* totals, cudaStream_t st) {
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorInvalidDevice;
-  // Steps per pass: the fewest microseconds in all, for the last ones (up to
-  // TAIL) exactly, before them passes of the cheapest kind per step.
-  constexpr int TAIL = 12;
-  TemporalPlan plan[MOST + 1];
-  double us[MOST + 1] = {0.0, single_us(s)};
-  int cheapest = 1;
-  const bool wide = s.nx >= (1 << 30) || s.ny >= (1 << 30);  // 32-bit rows and columns
-  for (int T = 2; T <= MOST && T <= nsteps; ++T) {
-    if (!wide) plan[T] = plan_temporal(s, T, sms);
-    us[T] = plan[T].us;
-    if (us[T] / T < us[cheapest] / cheapest) cheapest = T;
-  }
-  int left = nsteps, passes = 0;
-  double total = 0.0;
-  int head = 0;  // passes of `cheapest` steps before the tail
-  if (left > TAIL) {
-    head = (left - TAIL + cheapest - 1) / cheapest;
-    left -= head * cheapest;
-    total += head * us[cheapest];
-  }
-  double cost[TAIL + 1] = {0.0};
-  int first[TAIL + 1] = {0};
-  for (int n = 1; n <= left; ++n) {
-    cost[n] = 1e30;
-    for (int T = 1; T <= MOST && T <= n; ++T)
-      if (cost[n - T] + us[T] < cost[n]) cost[n] = cost[n - T] + us[T], first[n] = T;
-  }
-  total += cost[left];
-  passes = head;
-  for (int n = left; n > 0; n -= first[n]) ++passes;
-
-  const ResidentPlan rp = plan_resident(s, nsteps);
-  if (rp.C && resident_us(s, rp, nsteps) < total) {
-    const ResidentArgs a{fin, fout, s, tau, taus, 0.0f, nsteps, rp.rows};
-    return resident<false>(a, rp, st);
-  }
-  // ping-pong so that the last pass lands in fout
-  const float* src = fin;
-  for (int k = 0; k < passes; ++k) {
-    const int T = k < head ? cheapest : first[left];
-    if (k >= head) left -= T;
-    float* dst = (passes - k) % 2 == 1 ? fout : ftmp;
-    cudaError_t e = cudaSuccess;
-    switch (T) {
-      case 1: e = launch_bgk_step(src, dst, s, tau, taus, nullptr, st); break;
-      case 2: e = temporal<2>(src, dst, s, tau, taus, plan[2], st); break;
-      case 3: e = temporal<3>(src, dst, s, tau, taus, plan[3], st); break;
-      default: e = temporal<4>(src, dst, s, tau, taus, plan[4], st); break;
+  const bool cap = is_captured(st);
+  const StepsPlan all = plan_steps(s, nsteps, sms, cap);
+  if (totals) {
+    const double n = (double)s.nb * s.ny * s.nx;
+    const StepsPlan but_one = plan_steps(s, nsteps - 1, sms, cap);
+    const double blocks = (double)bgk_step_blocks(ftmp, fout, s);
+    if (but_one.us + single_us(s, cap) + fused_totals_us(blocks) < all.us + moments_us(n)) {
+      const cudaError_t e = run_steps(but_one, fin, ftmp, fout, s, tau, taus, nsteps - 1, st);
+      return e != cudaSuccess ? e : launch_bgk_step(ftmp, fout, s, tau, taus, totals, st);
     }
-    if (e != cudaSuccess) return e;
-    src = dst;
   }
-  return cudaSuccess;
+  const cudaError_t e = run_steps(all, fin, fout, ftmp, s, tau, taus, nsteps, st);
+  return e != cudaSuccess || !totals
+             ? e
+             : launch_moments(fout, s, nullptr, nullptr, nullptr, totals, st);
 }
 
 // The channel has the resident form alone; its single-step kernel takes 4.2 a
-// launch, 16.7e-6 per node.
-bool channel_steps_fit(const Shape& s, int nsteps) {
-  const ResidentPlan rp = plan_resident(s, nsteps);
-  const double single = std::max(4.2, 16.7e-6 * (double)s.nb * s.ny * s.nx);
-  return rp.C != 0 && 1.1 * resident_us(s, rp, nsteps) < 4.0 + nsteps * single;
+// launch (and 4 for the first; captured 2.5), 16.7e-6 per node.
+bool channel_steps_fit(const Shape& s, int nsteps, cudaStream_t st) {
+  const bool cap = is_captured(st);
+  const ResidentPlan rp = plan_resident(s, nsteps, true, cap);
+  const double n = (double)s.nb * s.ny * s.nx;
+  const double singles = cap ? nsteps * std::max({2.5, 2.2 + 15.5e-6 * n, 16.7e-6 * n})
+                             : 4.0 + nsteps * std::max(4.2, 16.7e-6 * n);
+  return rp.C != 0 && 1.1 * resident_us(s, rp, nsteps, true, cap) < singles;
 }
 
 cudaError_t launch_channel_steps(const float* fin, float* fout, const Shape& s, float tau,
                                  const float* taus, float gx, int nsteps, cudaStream_t st) {
-  const ResidentPlan rp = plan_resident(s, nsteps);
+  const ResidentPlan rp = plan_resident(s, nsteps, true, is_captured(st));
   if (!rp.C) return cudaErrorInvalidValue;
   const ResidentArgs a{fin, fout, s, tau, taus, gx, nsteps, rp.rows};
   return resident<true>(a, rp, st);
