@@ -241,9 +241,13 @@ def stream_ptr(stream=None):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
     # the current stream's handle, without the Stream object that
-    # torch.cuda.current_stream() builds around it
+    # torch.cuda.current_stream() builds around it where torch has the
+    # (private) function for that
     torch = _torch()
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def check(rc, what=""):
