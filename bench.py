@@ -2,13 +2,15 @@
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-One JSON line on rank 0.  A "step" is one lattice update of the
+One JSON line on stdout, on rank 0: the headline, short enough to be read whole
+from the end of a log; the full record of the run (the GNN workloads, training,
+tables, sweeps) goes to stderr and to the --log file.  A "step" is one lattice update of the
 Taylor-Green workload 4096 x 4096 (periodic, FP32 SoA populations, u0 = 0.05,
 k = 2 pi / 4096), timed with CUDA events on the stream the kernels run on;
 `value` is million lattice-node updates per second (MLUPS) over all ranks.
 Each rank advances its own lattice (weak scaling, no collective on the data
 path).  The GNN-LBM step on the 1024 x 1024 TGV (Re = 1000) is measured in
-the same run and reported beside it under "gnn".
+the same run and reported beside it under "gnn" (a summary in the headline).
 
 `--impl reference` times the FP64 CPU oracle (the slow, obviously-correct
 restatement of the method) on the host cores, one bounded sub-lattice per
@@ -97,6 +99,24 @@ def _src_sha(name):
 
 def _re(tau, n=N_SIDE, u0=U0):
     return u0 * n / ((tau - 0.5) / 3.0)
+
+
+def headline(out):
+    """The stdout line of a full record: every field but the long ones, with the
+    GNN workloads' rates in the place of their records."""
+    h = {k: v for k, v in out.items() if k not in ("tau_sweep", "tgv64")}
+    if "timing" in h:
+        h["timing"] = {k: v for k, v in h["timing"].items() if not isinstance(v, (list, tuple))}
+    if "cpu_baseline" in h:
+        h["cpu_baseline"] = {k: v for k, v in h["cpu_baseline"].items() if not isinstance(v, dict)}
+    if "gnn" in h:
+        g = out["gnn"]
+        pick = {"xavier": ("workload", "mlups_gnn", "ms_per_step_gnn"),
+                "training": ("workload", "ms_per_fused_train_step"),
+                "mlp_fused": ("workload", "mlups_gnn_mlp", "ms_per_step_gnn_mlp"),
+                "batch": ("workload", "mlups_total", "ms_per_step")}
+        h["gnn"] = {name: {k: g[name].get(k) for k in keys} for name, keys in pick.items() if name in g}
+    return h
 
 
 class ClockSampler:
@@ -1281,7 +1301,7 @@ def main():
                     help="time one kernel family only (profiling runs)")
     ap.add_argument("--side", type=int, default=N_SIDE, help="lattice side for --only runs")
     ap.add_argument("--log", default=None,
-                    help="also append the JSON line to this JSON-lines file (rank 0)")
+                    help="also append the full record to this JSON-lines file (rank 0)")
     args = ap.parse_args()
     if args.warmup < 3:
         ap.error("--warmup must be >= 3")
@@ -1302,7 +1322,8 @@ def main():
         out = run_ours(args, rank, world, local_rank)
     if out is not None and rank == 0:
         line = json.dumps(_finite(out), allow_nan=False)
-        print(line, flush=True)
+        print("full record: " + line, file=sys.stderr, flush=True)
+        print(json.dumps(_finite(headline(out)), allow_nan=False), flush=True)
         if args.log:
             d = os.path.dirname(os.path.abspath(args.log))
             os.makedirs(d, exist_ok=True)
