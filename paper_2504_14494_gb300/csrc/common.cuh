@@ -48,8 +48,8 @@ __device__ __forceinline__ void raise_status(unsigned* w, unsigned bits) { atomi
 // Bounds-checked builds (-DLBM_BOUNDS_CHECK, liblbmgnn_checked.so): a computed
 // gather index outside [lo, hi) raises ST_BOUNDS and is replaced by lo, so
 // the access stays inside the buffer and the run goes on; the regular build
-// compiles the check away.  (The pool offers no memory checker; this build
-// plus small cases and the oracle stand in for one.)
+// compiles the check away.  (This build, small cases and the oracle stand in
+// for a memory checker.)
 __device__ __forceinline__ int64_t checked(int64_t i, int64_t lo, int64_t hi, unsigned* stw) {
 #ifdef LBM_BOUNDS_CHECK
   if (i < lo || i >= hi) {

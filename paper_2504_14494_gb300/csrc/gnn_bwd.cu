@@ -952,8 +952,9 @@ __global__ void __launch_bounds__(256, LBM_EB_CTAS) gnn_encode_bwd_kernel(
 // ---------------------------------------------------------------------------
 // Sum of the per-CTA gradient rows, from the first to the last; every kernel
 // writes its own parameters' columns in as many rows as it has CTAs.  A thread
-// per parameter; bound by the latency of its loads, of which 32 rows are in
-// flight (26 us for 512 rows before, most of them empty; 6 for 128 rows).
+// per parameter; bound by the latency of its loads, which are independent
+// within batches of 32 rows (as many in flight as its 30 registers hold; 26 us
+// for 512 rows before, most of them empty; 6 for 128 rows).
 // accumulate: add to the gradient already in grad (the steps of a rollout).
 struct GradRows {
   int enc, edge, node, head;
