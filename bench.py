@@ -47,24 +47,23 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
     #     --clock-control none -k regex:bgk_step_x4 -s 3 -c 1
     #     python bench.py --only bgk --steps 10 --warmup 3      (4096 x 4096, one launch)
-    "bgk_step_x4": {"bytes_per_launch": 604054528 + 547321088,
-                    "src_sha": "75175dfa13fa1003a94d217d10ae26bfeaf1caf2b0033fe04d22f926f7b425a7"},
+    "bgk_step_x4": {"bytes_per_launch": 604035328 + 547279360,
+                    "src_sha": "c361951bbca67452362ae7d5185e3edf6334a82adc138553e6b85d5e3f24f94f"},
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
-    #     --clock-control none -k regex:"gnn_(mlp_step|round)_kernel" -s 4 -c 4
+    #     --clock-control none -k regex:"gnn_(step_first|round)_kernel" -s 3 -c 3
     #     python bench.py --only gnn --steps 20 --warmup 3   (one GNN-LBM step, 1024 x 1024:
-    #     the MLP-only kernel returning at once, the fused encoder, 2 rounds; key files
-    #     gnn_fwd.cu and gnn_mlp.cu)
-    "lbm_step_gnn": {"bytes_per_launch": 50432 + (37957376 + 204766976) + (269698048 + 213554176)
-                     + (306590208 + 25459456), "nodes": 1024 * 1024,
+    #     the fused encoder, 2 rounds; key files gnn_fwd.cu and gnn_mlp.cu)
+    "lbm_step_gnn": {"bytes_per_launch": (38159104 + 208859904) + (269575680 + 213989632)
+                     + (306580992 + 25687808), "nodes": 1024 * 1024,
                      "file": ["gnn_fwd.cu", "gnn_mlp.cu"],
-                     "src_sha": ["9d25ba2e220528efef29d6d0450ede2be182d67d0e211582c3843e5a0c9355be",
-                                 "f4c35f4c20b57a0feca1e66b043ceb113a26a00364f07f524735a77ff9b9f640"]},
+                     "src_sha": ["86e1c5868386e4054fb61fdaa400a213954ffb464747652614837dbfe7c89f15",
+                                 "41f9d20607b65813e446e6c6f6830da66e64035e4d5e69bcb07ada862437133c"]},
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
     #     --clock-control none -k regex:gnn_mlp_step -s 3 -c 1
     #     python bench.py --only mlp --side 4096 --steps 10 --warmup 3   (one fused step)
-    "gnn_mlp_step_kernel": {"bytes_per_launch": 604143616 + 555024640, "nodes": 4096 * 4096,
+    "gnn_mlp_step_kernel": {"bytes_per_launch": 604060416 + 554683904, "nodes": 4096 * 4096,
                             "file": "gnn_mlp.cu",
-                            "src_sha": "f4c35f4c20b57a0feca1e66b043ceb113a26a00364f07f524735a77ff9b9f640"},
+                            "src_sha": "41f9d20607b65813e446e6c6f6830da66e64035e4d5e69bcb07ada862437133c"},
 }
 
 
@@ -589,7 +588,7 @@ def gnn_bench(args, L, dev, stream, side=GNN_SIDE, only=False, theta=None, label
                               f"message sequence, MUFU tanh bound; microbench/fp16_rate.cu)",
                 "achieved": round(ach, 1), "peak": round(peak, 1), "unit": "G edge-feature GELU/s",
                 "frac": round(ach / peak, 4), "traffic": traffic,
-                "traffic_note": "DRAM bytes of one step (fused encoder, 2 rounds and the MLP-only kernel returning at once), ncu"},
+                "traffic_note": "DRAM bytes of one step (fused encoder, 2 rounds), ncu"},
             "weights": label,
             "steps_timed": kk, "steps_run": args.warmup + kk,
             "mlups_gnn": res["gnn"]["mlups"], "mlups_bgk_same_lattice": res["bgk"]["mlups"],
